@@ -2970,14 +2970,16 @@ int cvsadc_create(cvsadc_ctx** ctx, int device, void* cuda_stream) {
     init_kernel_attributes();
     init_gemm_attributes();
     c->s_kpart.ensure((size_t)8 << 20 << 4);  // 8 Mi complex = 128 MB
-    c->err.ensure(256);
-    CVS_CUDA(cudaMemset(c->err.p, 0, 256));
     if (cuda_stream) {
       c->stream = (cudaStream_t)cuda_stream;
     } else {
       CVS_CUDA(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
       c->own_stream = true;
     }
+    // cleared on the context's own stream: a memset on the default stream is
+    // not ordered before the error check that ends this call
+    c->err.ensure(256);
+    CVS_CUDA(cudaMemsetAsync(c->err.p, 0, 256, c->stream));
   });
   if (rc != CVSADC_OK) {
     delete c;

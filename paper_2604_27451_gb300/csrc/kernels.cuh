@@ -15,7 +15,6 @@ void zgemm_f64(cudaStream_t s, int M, int N, int K, double alpha, View A,
 // C(m, n) = sum_z part[z][m][n] + beta * C(m, n), part dense [nz][M][N]
 void splitk_reduce(cudaStream_t s, int M, int N, int nz, const cplx* part,
                    double beta, View C);
-void init_gemm_attributes();
 
 // Same contract on the tcgen05 tensor cores: A and B are split into bf16
 // parts, nprod = 3 (hi/lo, BF16x3) or 6 (hi/mid/lo, BF16x6) products per

@@ -2968,7 +2968,6 @@ int cvsadc_create(cvsadc_ctx** ctx, int device, void* cuda_stream) {
   c->device = device;
   int rc = guarded(c, [&] {
     init_kernel_attributes();
-    init_gemm_attributes();
     c->s_kpart.ensure((size_t)8 << 20 << 4);  // 8 Mi complex = 128 MB
     if (cuda_stream) {
       c->stream = (cudaStream_t)cuda_stream;

@@ -1,12 +1,18 @@
 // FP64 complex Hermitian eigensolver: cyclic Jacobi with the round-robin
 // (Brent-Luk) pair ordering, so that the n/2 rotations of one step act on
-// disjoint index pairs and are applied in parallel by one CTA.  Used for
-// the Davidson subspace matrix and for the MP2 vv density and the
-// truncated Fock block of the frozen-natural-spinor step (Eqs. 17 and 19).
+// disjoint index pairs.  Used for the Davidson subspace matrix, for the MP2
+// vv density and the truncated Fock block of the frozen-natural-spinor step
+// (Eqs. 17 and 19) and for the Schur-complement preconditioner.
 //
-// Each rotation zeroes a_pq with the unitary J = [[c, s e], [-s conj(e), c]]
-// (e = a_pq/|a_pq|, t = tan(theta) = sgn(tau)/(|tau| + sqrt(1+tau^2)),
-// tau = (a_qq - a_pp)/(2|a_pq|)): A <- J^H A J, V <- V J.
+// A rotation is the unitary J = [[c, s], [-conj(s), c]] on the pair (p, q):
+// A <- J^H A J, V <- V J, with s = c t a_pq / |a_pq|, c = (1 + t^2)^-1/2,
+// t = sgn(tau) / (|tau| + sqrt(1 + tau^2)), tau = (a_qq - a_pp) / (2 |a_pq|).
+//
+// Up to SMALL_N indices one CTA runs the whole solve; above, every step of a
+// sweep is one grid-wide launch (jstep_kernel).
+#include <cmath>
+#include <vector>
+
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -15,8 +21,7 @@ namespace cvs {
 namespace {
 
 __global__ void __launch_bounds__(1024)
-    jacobi_kernel(cplx* A, int n, double* w, cplx* V, int max_sweeps,
-                  double* info) {
+    jacobi_kernel(cplx* A, int n, double* w, cplx* V, int max_sweeps) {
   extern __shared__ char smem[];
   const int np = (n + 1) & ~1;
   const int half = np / 2;
@@ -171,22 +176,261 @@ __global__ void __launch_bounds__(1024)
   }
   __syncthreads();
   for (int64_t e = tid; e < (int64_t)n * n; e += nt) V[e] = A[e];
-  if (tid == 0 && info) {
-    info[0] = sweep;
-    info[1] = ratio;
+}
+
+// ------------------------------------------------------- one step per launch
+// Pairs of step s of the round-robin tournament over np (even) positions:
+// position 0 stays, the others rotate by one per step.  q = n (odd n) is the
+// bye: the pair's one index is left alone.
+__device__ __forceinline__ void rr_pair(int k, int np, int s, int& p, int& q) {
+  auto pos = [&](int kk) {
+    int t = kk - 1 - s;  // > -2 np
+    t += t < 0 ? np - 1 : 0;
+    t += t < 0 ? np - 1 : 0;
+    return kk == 0 ? 0 : 1 + t;
+  };
+  p = pos(k);
+  q = pos(np - 1 - k);
+  if (p > q) {
+    const int t = p;
+    p = q;
+    q = t;
   }
+}
+
+// the rotation of a_pq, skipped for |a_pq| <= 1e-18 sqrt(|a_pp a_qq|)
+__device__ __forceinline__ void rotation(cplx apq, double app, double aqq, double& c, cplx& sv) {
+  c = 1.0;
+  sv = cmake(0.0, 0.0);
+  const double r = hypot(apq.x, apq.y);
+  if (!(r > 1e-300 && r > 1e-18 * sqrt(fabs(app * aqq)))) return;
+  const double tau = (aqq - app) / (2.0 * r);
+  const double t = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
+  c = 1.0 / sqrt(1.0 + t * t);
+  const double sn = t * c;
+  sv = cmake(sn * apq.x / r, sn * apq.y / r);
+}
+
+// One step: An = J^H A J and V = V J for all pairs of the step.
+//
+// What bounds it: the FP64 pipes (two FMAs per SM and cycle), launch and
+// latency at small n.  A is only read, so a block takes a tile of JT x JT
+// pairs, computes their rotations and both sides of its (2 JT)^2 elements in
+// one pass (48 FP64 operations per 2 x 2 block, ~150 per rotation) and
+// writes them to An: one launch a step and one pass over A instead of three
+// and two.  Blocks from na on rotate JT pairs of columns of VR rows of V.
+// The rotations are worked out again in every block, so the larger tile
+// takes over where blocks outnumber the SMs.
+// A launch a step, measured against three: n = 600 24 us (33 us),
+// n = 240 11.6 us (20 us), n = 200 against one CTA 11 us (~190 us).
+template <int JT, int VR>
+__global__ void __launch_bounds__(JT * JT)
+    jstep_kernel(const cplx* __restrict__ A, cplx* __restrict__ An, cplx* __restrict__ V,
+                 int n, int np, int s, int nt, int na) {
+  __shared__ double cc[2 * JT];
+  __shared__ cplx se[2 * JT];
+  __shared__ int ip[2 * JT], iq[2 * JT];
+  const int tid = threadIdx.x, ti = tid / JT, tj = tid % JT;
+  const bool vblk = (int)blockIdx.x >= na;
+  const int blk = vblk ? (int)blockIdx.x - na : (int)blockIdx.x;
+  const int tk = blk / nt, tl = blk % nt;  // tk of a V block: its tile of rows
+  // pairs of the tile's columns at [0, JT), of its rows at [JT, 2 JT)
+  if (tid < 2 * JT) {
+    const int k = (tid < JT ? tl : tk) * JT + tid % JT;
+    int p = n, q = n;
+    if (k < np / 2 && !(vblk && tid >= JT)) rr_pair(k, np, s, p, q);
+    double c = 1.0;
+    cplx sv = cmake(0.0, 0.0);
+    if (q < n)
+      rotation(A[(int64_t)p * n + q], A[(int64_t)p * n + p].x, A[(int64_t)q * n + q].x, c, sv);
+    cc[tid] = c;
+    se[tid] = sv;
+    ip[tid] = p;
+    iq[tid] = q;
+  }
+  __syncthreads();
+  const int pl = ip[tj], ql = iq[tj];
+  const double cl = cc[tj];
+  const cplx sl = se[tj];
+  if (vblk) {
+    if (ql >= n || (sl.x == 0.0 && sl.y == 0.0)) return;
+    for (int r = tk * VR + ti; r < min(n, (tk + 1) * VR); r += JT) {
+      cplx* v = V + (int64_t)r * n;
+      const cplx vp = v[pl], vq = v[ql];
+      v[pl] = csub(cscale(vp, cl), cmul(cconj(sl), vq));
+      v[ql] = cadd(cmul(sl, vp), cscale(vq, cl));
+    }
+    return;
+  }
+  const int pk = ip[JT + ti], qk = iq[JT + ti];
+  const double ck = cc[JT + ti];
+  const cplx sk = se[JT + ti];
+  auto get = [&](int r, int c) {
+    return r < n && c < n ? A[(int64_t)r * n + c] : cmake(0.0, 0.0);
+  };
+  auto put = [&](int r, int c, cplx v) {
+    if (r < n && c < n) An[(int64_t)r * n + c] = v;
+  };
+  cplx a = get(pk, pl), b = get(pk, ql), c = get(qk, pl), d = get(qk, ql);
+  if (sk.x != 0.0 || sk.y != 0.0) {  // rows: p' = c p - s q, q' = conj(s) p + c q
+    const cplx a0 = a, b0 = b;
+    a = csub(cscale(a0, ck), cmul(sk, c));
+    c = cadd(cmul(cconj(sk), a0), cscale(c, ck));
+    b = csub(cscale(b0, ck), cmul(sk, d));
+    d = cadd(cmul(cconj(sk), b0), cscale(d, ck));
+  }
+  if (sl.x != 0.0 || sl.y != 0.0) {  // columns: p' = c p - conj(s) q, q' = s p + c q
+    const cplx a0 = a, c0 = c;
+    a = csub(cscale(a0, cl), cmul(cconj(sl), b));
+    b = cadd(cmul(sl, a0), cscale(b, cl));
+    c = csub(cscale(c0, cl), cmul(cconj(sl), d));
+    d = cadd(cmul(sl, c0), cscale(d, cl));
+  }
+  put(pk, pl, a);
+  put(pk, ql, b);
+  put(qk, pl, c);
+  put(qk, ql, d);
+}
+
+__global__ void jidentity_kernel(cplx* V, int n) {
+  const int64_t total = (int64_t)n * n;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
+       e += (int64_t)gridDim.x * blockDim.x)
+    V[e] = cmake(e / n == e % n ? 1.0 : 0.0, 0.0);
+}
+
+// per-block partial sums of the off-diagonal and total squared modulus
+constexpr int JPART = 304;
+__global__ void __launch_bounds__(256)
+    joffnorm_kernel(const cplx* __restrict__ A, int n, double* __restrict__ part) {
+  __shared__ double so[8], st[8];
+  double off = 0.0, tot = 0.0;
+  const int64_t total = (int64_t)n * n;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const cplx a = A[e];
+    const double m2 = a.x * a.x + a.y * a.y;
+    tot += m2;
+    if (e / n != e % n) off += m2;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    off += __shfl_xor_sync(0xffffffffu, off, o);
+    tot += __shfl_xor_sync(0xffffffffu, tot, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    so[threadIdx.x >> 5] = off;
+    st[threadIdx.x >> 5] = tot;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < 8; ++q) {
+      off += so[q];
+      tot += st[q];
+    }
+    part[2 * blockIdx.x] = off;
+    part[2 * blockIdx.x + 1] = tot;
+  }
+}
+
+// rank[i] = place of eigenvalue i in ascending order, w sorted
+__global__ void jrank_kernel(const cplx* __restrict__ A, int n, double* __restrict__ w,
+                             int* __restrict__ rank) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const double wi = A[(int64_t)i * n + i].x;
+    int r = 0;
+    for (int j = 0; j < n; ++j) {
+      const double wj = A[(int64_t)j * n + j].x;
+      r += (wj < wi) || (wj == wi && j < i);
+    }
+    w[r] = wi;
+    rank[i] = r;
+  }
+}
+
+__global__ void jcolumns_kernel(const cplx* __restrict__ V, int n, const int* __restrict__ rank,
+                                cplx* __restrict__ U) {
+  const int64_t total = (int64_t)n * n;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
+       e += (int64_t)gridDim.x * blockDim.x)
+    U[e / n * n + rank[e % n]] = V[e];
 }
 
 }  // namespace
 
-void jacobi_eigh(cudaStream_t s, cplx* A, int n, double* w, cplx* Vec,
-                 int max_sweeps, double* info_dev) {
+// The one-CTA solve runs at an SM's two FP64 FMAs per cycle (18 n^3 a
+// sweep); a step launch costs ~3 us.  They meet near n = 24 (one sweep: 60
+// against 70 us).
+constexpr int SMALL_N = 24;
+
+// scratch of jacobi_eigh_grid: a second A, partial sums, ranks
+static size_t grid_work_bytes(int n) {
+  return (size_t)n * n * sizeof(cplx) + 2 * JPART * sizeof(double) +
+         ((size_t)n * sizeof(int) + 15) / 16 * 16;
+}
+size_t jacobi_work_bytes(int n) {
+  return (size_t)n * n * sizeof(cplx) + grid_work_bytes(n);
+}
+
+int jacobi_eigh_grid(cudaStream_t s, cplx* A, int n, double* w, cplx* U, cplx* V, void* work,
+                     int max_sweeps, double tol, double floor) {
+  CVS_REQUIRE(n >= 1 && n <= 16384, -1, "jacobi_eigh_grid: n out of range");
+  cplx* bufs[2] = {A, (cplx*)work};
+  double* part = (double*)((cplx*)work + (size_t)n * n);
+  int* rank = (int*)(part + 2 * JPART);
+  const int np = (n + 1) & ~1;
+  // 8 x 8 pairs give 345 blocks at n = 240 (2.3 per SM), 16 x 16 give 456 at
+  // n = 600 with a quarter of the repeated rotations
+  const bool large = n >= 400;
+  const int jt = large ? 16 : 8, vr = large ? 128 : 32;
+  const int nt = (np / 2 + jt - 1) / jt;
+  const int na = nt * nt;
+  const unsigned grid = (unsigned)(na + nt * ((n + vr - 1) / vr));
+  jidentity_kernel<<<grid1d((int64_t)n * n, 256), 256, 0, s>>>(V, n);
+  CVS_CHECK_LAUNCH();
+  int sweep = 0, cur = 0;
+  double prev = 1e300;
+  std::vector<double> hp(2 * JPART);
+  for (; sweep < max_sweeps; ++sweep) {
+    joffnorm_kernel<<<JPART, 256, 0, s>>>(bufs[cur], n, part);
+    CVS_CHECK_LAUNCH();
+    CVS_CUDA(cudaMemcpyAsync(hp.data(), part, hp.size() * sizeof(double),
+                             cudaMemcpyDeviceToHost, s));
+    CVS_CUDA(cudaStreamSynchronize(s));
+    double off = 0.0, tot = 0.0;
+    for (int b = 0; b < JPART; ++b) {
+      off += hp[2 * b];
+      tot += hp[2 * b + 1];
+    }
+    const double ratio = tot > 0.0 ? std::sqrt(off / tot) : 0.0;
+    // converged, or stalled at the rounding level of the largest entries
+    if (ratio < tol || (ratio < floor && ratio > 0.5 * prev)) break;
+    prev = ratio;
+    for (int st = 0; st < np - 1; ++st, cur ^= 1) {
+      auto* step = large ? jstep_kernel<16, 128> : jstep_kernel<8, 32>;
+      step<<<grid, jt * jt, 0, s>>>(bufs[cur], bufs[cur ^ 1], V, n, np, st, nt, na);
+      CVS_CHECK_LAUNCH();
+    }
+  }
+  jrank_kernel<<<(n + 127) / 128, 128, 0, s>>>(bufs[cur], n, w, rank);
+  CVS_CHECK_LAUNCH();
+  jcolumns_kernel<<<grid1d((int64_t)n * n, 256), 256, 0, s>>>(V, n, rank, U);
+  CVS_CHECK_LAUNCH();
+  return sweep;
+}
+
+void jacobi_eigh(cudaStream_t s, cplx* A, int n, double* w, cplx* Vec, int max_sweeps,
+                 void* work) {
   CVS_REQUIRE(n >= 1 && n <= 4096, -1, "jacobi_eigh: n out of range");
-  int np = (n + 1) & ~1;
-  int half = np / 2;
+  if (n > SMALL_N) {
+    cplx* V = (cplx*)work;
+    jacobi_eigh_grid(s, A, n, w, Vec, V, V + (size_t)n * n, max_sweeps, 1e-15, 1e-13);
+    return;
+  }
+  const int np = (n + 1) & ~1, half = np / 2;
   size_t sh = (size_t)(np + 2) * sizeof(int) + (size_t)(half + 2) * sizeof(double) +
               (size_t)half * sizeof(cplx) + 64;
-  jacobi_kernel<<<1, 1024, sh, s>>>(A, n, w, Vec, max_sweeps, info_dev);
+  jacobi_kernel<<<1, 1024, sh, s>>>(A, n, w, Vec, max_sweeps);
   CVS_CHECK_LAUNCH();
 }
 

@@ -191,11 +191,19 @@ void herm_project(cudaStream_t s, cplx* G, int n, int64_t nmat);
 
 // ---------------------------------------------------- Jacobi (FP64)
 // Hermitian eigensolver: A [n][n] row-major (destroyed), eigenvalues w
-// ascending, eigenvectors as columns of Vec [n][n].  One CTA, cyclic
-// round-robin (Brent-Luk) ordering; at most max_sweeps sweeps.
-// info_dev[0] = sweeps used (as double), [1] = final off-norm ratio.
+// ascending, eigenvectors as columns of Vec [n][n]; cyclic Jacobi with
+// round-robin (Brent-Luk) ordering, until the off-diagonal norm is below
+// 1e-15 of the total or no longer falls, at most max_sweeps sweeps.  work:
+// jacobi_work_bytes(n) bytes.
+size_t jacobi_work_bytes(int n);
 void jacobi_eigh(cudaStream_t s, cplx* A, int n, double* w, cplx* Vec,
-                 int max_sweeps, double* info_dev);
+                 int max_sweeps, void* work);
+// The same over the whole grid for any n: A -> w, U, with V [n][n] and work
+// (jacobi_work_bytes(n) less one n x n) as scratch; until the off-diagonal
+// norm is below tol of the total, or below floor and no longer halving.
+// Returns the sweeps done.
+int jacobi_eigh_grid(cudaStream_t s, cplx* A, int n, double* w, cplx* U, cplx* V, void* work,
+                     int max_sweeps, double tol, double floor);
 
 // Schur-complement preconditioner (schur_kernels.cu)
 void h_assemble(cudaStream_t s, const cplx* hc1, const cplx* hc2, int nc,
@@ -211,9 +219,6 @@ void h_weight(cudaStream_t s, const cplx* h, int j, int nc, int nw, int nv,
 void schur_assemble(cudaStream_t s, const cplx* M11, const cplx* C11,
                     const cplx* C12, const cplx* h, int nc, int nw, int nv,
                     const double* eps, double theta, cplx* S22, cplx* S);
-int jacobi_eigh_parallel(cudaStream_t s, cplx* A, int n, double* w, cplx* U,
-                         cplx* V, double* part, double* cc, cplx* se,
-                         int max_sweeps);
 void fold_doubles(cudaStream_t s, const cplx* R, const cplx* U2,
                   const double* theta, int k, int64_t N, int64_t N1, int nc,
                   int nw, int nv, const double* eps, bool zero_singles,

@@ -17,10 +17,7 @@
 // (12) as a batched GEMM; (22) and (23) involve only the small <Kb||Ij>
 // tensor and are summed here while S is assembled.
 //
-// Also here: a Jacobi eigensolver for Hermitian matrices too large for one
-// CTA (the same cyclic round-robin rotations as jacobi.cu, each step split
-// into three grid-wide launches), and the elementwise steps of applying
-// the preconditioner.
+// Also here: the elementwise steps of applying the preconditioner.
 #include <algorithm>
 #include <vector>
 
@@ -251,138 +248,6 @@ __global__ void schur_assemble_kernel(const cplx* __restrict__ M11,
     val.x += sr;
     val.y += si;
     S[e] = val;
-  }
-}
-
-// ------------------------------------------------------ parallel Jacobi
-// Pairs of step s of the round-robin tournament over np (even) positions:
-// position 0 stays, the others rotate by one per step.
-__device__ __forceinline__ void rr_pair(int k, int np, int s, int& p, int& q) {
-  auto pos = [&](int kk) {
-    return kk == 0 ? 0 : 1 + ((kk - 1 - s) % (np - 1) + (np - 1)) % (np - 1);
-  };
-  p = pos(k);
-  q = pos(np - 1 - k);
-  if (p > q) {
-    const int t = p;
-    p = q;
-    q = t;
-  }
-}
-
-__global__ void pj_identity_kernel(cplx* V, int n) {
-  const int64_t total = (int64_t)n * n;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x)
-    V[e] = cmake(e / n == e % n ? 1.0 : 0.0, 0.0);
-}
-
-__global__ void pj_params_kernel(const cplx* __restrict__ A, int n, int np,
-                                 int s, double* __restrict__ cc,
-                                 cplx* __restrict__ se) {
-  const int half = np / 2;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < half;
-       k += gridDim.x * blockDim.x) {
-    int p, q;
-    rr_pair(k, np, s, p, q);
-    double c = 1.0;
-    cplx sv = cmake(0, 0);
-    if (q < n) {
-      const cplx apq = A[(int64_t)p * n + q];
-      const double r = hypot(apq.x, apq.y);
-      const double app = A[(int64_t)p * n + p].x, aqq = A[(int64_t)q * n + q].x;
-      if (r > 1e-300 && r > 1e-18 * sqrt(fabs(app * aqq))) {
-        const double tau = (aqq - app) / (2.0 * r);
-        const double t = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-        c = 1.0 / sqrt(1.0 + t * t);
-        const double sn = t * c;
-        sv = cmake(sn * apq.x / r, sn * apq.y / r);
-      }
-    }
-    cc[k] = c;
-    se[k] = sv;
-  }
-}
-
-// rows p, q of A: A <- J^H A
-__global__ void pj_rows_kernel(cplx* A, int n, int np, int s,
-                               const double* __restrict__ cc,
-                               const cplx* __restrict__ se) {
-  const int half = np / 2;
-  const int64_t total = (int64_t)half * n;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int k = e / n, col = e % n;
-    int p, q;
-    rr_pair(k, np, s, p, q);
-    if (q >= n) continue;
-    const cplx sv = se[k];
-    if (sv.x == 0.0 && sv.y == 0.0) continue;
-    const double c = cc[k];
-    const cplx ap = A[(int64_t)p * n + col], aq = A[(int64_t)q * n + col];
-    A[(int64_t)p * n + col] = csub(cscale(ap, c), cmul(sv, aq));
-    A[(int64_t)q * n + col] = cadd(cmul(cconj(sv), ap), cscale(aq, c));
-  }
-}
-
-// columns p, q of A and V: A <- A J, V <- V J
-__global__ void pj_cols_kernel(cplx* A, cplx* V, int n, int np, int s,
-                               const double* __restrict__ cc,
-                               const cplx* __restrict__ se) {
-  const int half = np / 2;
-  const int64_t total = (int64_t)half * n;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int k = e / n, row = e % n;
-    int p, q;
-    rr_pair(k, np, s, p, q);
-    if (q >= n) continue;
-    const cplx sv = se[k];
-    if (sv.x == 0.0 && sv.y == 0.0) continue;
-    const double c = cc[k];
-    const cplx ap = A[(int64_t)row * n + p], aq = A[(int64_t)row * n + q];
-    A[(int64_t)row * n + p] = csub(cscale(ap, c), cmul(cconj(sv), aq));
-    A[(int64_t)row * n + q] = cadd(cmul(sv, ap), cscale(aq, c));
-    const cplx vp = V[(int64_t)row * n + p], vq = V[(int64_t)row * n + q];
-    V[(int64_t)row * n + p] = csub(cscale(vp, c), cmul(cconj(sv), vq));
-    V[(int64_t)row * n + q] = cadd(cmul(sv, vp), cscale(vq, c));
-  }
-}
-
-// per-block partial sums of the off-diagonal and total squared modulus
-__global__ void pj_offnorm_kernel(const cplx* __restrict__ A, int n,
-                                  double* __restrict__ part) {
-  double off = 0.0, tot = 0.0;
-  const int64_t total = (int64_t)n * n;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const cplx a = A[e];
-    const double m2 = a.x * a.x + a.y * a.y;
-    tot += m2;
-    if (e / n != e % n) off += m2;
-  }
-  off = sum_block(off);
-  tot = sum_block(tot);
-  if (threadIdx.x == 0) {
-    part[2 * blockIdx.x] = off;
-    part[2 * blockIdx.x + 1] = tot;
-  }
-}
-
-// ascending eigenvalues w and the matching columns of V into U
-__global__ void pj_sort_kernel(const cplx* __restrict__ A,
-                               const cplx* __restrict__ V, int n,
-                               double* __restrict__ w, cplx* __restrict__ U) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += gridDim.x * blockDim.x) {
-    const double wi = A[(int64_t)i * n + i].x;
-    int rank = 0;
-    for (int j = 0; j < n; ++j) {
-      const double wj = A[(int64_t)j * n + j].x;
-      rank += (wj < wi) || (wj == wi && j < i);
-    }
-    w[rank] = wi;
-    for (int r = 0; r < n; ++r) U[(int64_t)r * n + rank] = V[(int64_t)r * n + i];
   }
 }
 
@@ -664,52 +529,6 @@ void schur_assemble(cudaStream_t s, const cplx* M11, const cplx* C11,
   schur_assemble_kernel<<<grid1d(N1 * N1, 128), 128, 0, s>>>(
       M11, C11, C12, S22, h, nc, nw, nv, eps, theta, S);
   CVS_CHECK_LAUNCH();
-}
-
-// Eigen-decomposition A = U diag(w) U^H of a Hermitian n x n matrix (A is
-// overwritten; V is an n x n work matrix; part holds 2 * 304 doubles; cc,
-// se hold n/2 + 1 entries).  Sweeps until the off-diagonal norm falls below
-// 1e-13 of the total (at most max_sweeps); returns the sweeps done.
-int jacobi_eigh_parallel(cudaStream_t s, cplx* A, int n, double* w, cplx* U,
-                         cplx* V, double* part, double* cc, cplx* se,
-                         int max_sweeps) {
-  CVS_REQUIRE(n >= 1 && n <= 16384, -1, "jacobi_eigh_parallel: n out of range");
-  const int np = (n + 1) & ~1;
-  const int half = np / 2;
-  pj_identity_kernel<<<grid1d((int64_t)n * n, 256), 256, 0, s>>>(V, n);
-  CVS_CHECK_LAUNCH();
-  const unsigned gp = (unsigned)std::max(1, (half + 127) / 128);
-  const unsigned gr = grid1d((int64_t)half * n, 256);
-  int sweep = 0;
-  double prev = 1e300;
-  std::vector<double> hp(2 * 304);
-  for (; sweep < max_sweeps; ++sweep) {
-    pj_offnorm_kernel<<<304, 256, 0, s>>>(A, n, part);
-    CVS_CHECK_LAUNCH();
-    CVS_CUDA(cudaMemcpyAsync(hp.data(), part, hp.size() * sizeof(double),
-                             cudaMemcpyDeviceToHost, s));
-    CVS_CUDA(cudaStreamSynchronize(s));
-    double off = 0.0, tot = 0.0;
-    for (int b = 0; b < 304; ++b) {
-      off += hp[2 * b];
-      tot += hp[2 * b + 1];
-    }
-    const double ratio = tot > 0.0 ? std::sqrt(off / tot) : 0.0;
-    // converged, or stalled at the rounding level of the largest entries
-    if (ratio < 1e-10 || (ratio < 1e-7 && ratio > 0.5 * prev)) break;
-    prev = ratio;
-    for (int st = 0; st < np - 1; ++st) {
-      pj_params_kernel<<<gp, 128, 0, s>>>(A, n, np, st, cc, se);
-      CVS_CHECK_LAUNCH();
-      pj_rows_kernel<<<gr, 256, 0, s>>>(A, n, np, st, cc, se);
-      CVS_CHECK_LAUNCH();
-      pj_cols_kernel<<<gr, 256, 0, s>>>(A, V, n, np, st, cc, se);
-      CVS_CHECK_LAUNCH();
-    }
-  }
-  pj_sort_kernel<<<grid1d(n, 128), 128, 0, s>>>(A, V, n, w, U);
-  CVS_CHECK_LAUNCH();
-  return sweep;
 }
 
 void fold_doubles(cudaStream_t s, const cplx* R, const cplx* U2,

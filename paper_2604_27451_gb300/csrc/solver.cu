@@ -175,6 +175,7 @@ struct cvsadc_ctx {
   // Schur-complement preconditioner of the prepared problem
   DBuf sch_W, sch_g, sch_S, sch_U, sch_V, sch_lam, sch_C11, sch_C12, sch_work,
       sch_tmp, sch_th;
+  DBuf jac;  // scratch of the Jacobi eigensolver
   bool sch_on = false;
   // eigenvectors held in sch_U ([N1][sch_p] columns): all N1, or the lowest
   // SCHUR_PL for large singles spaces (the folded solver only)
@@ -208,7 +209,7 @@ struct cvsadc_ctx {
             &s_part, &s_small, &s_tc, &dv_V, &dv_W, &dv_X, &dv_AX, &dv_T,
             &dv_H,  &dv_A,  &dv_U,  &dv_w, &dv_misc, &sch_W, &sch_g,
             &sch_S, &sch_U, &sch_V, &sch_lam, &sch_C11, &sch_C12, &sch_work,
-            &sch_tmp, &sch_th, &fd_A, &fd_B, &fd_th, &fv_V, &fv_B, &fv_R, &fv_D,
+            &sch_tmp, &sch_th, &jac, &fd_A, &fd_B, &fd_th, &fv_V, &fv_B, &fv_R, &fv_D,
             &fv_MV, &fv_T, &fv_T2, &fv_small};
   }
   // give back every problem-sized buffer (the context stays usable)
@@ -372,6 +373,13 @@ void copyv(cvsadc_ctx* c, int M, int N, double alpha, View src, View dst) {
   check_view(src, M, N, 1, "copy src");
   check_view(dst, M, N, 1, "copy dst");
   copy_view(c->stream, M, N, alpha, src, dst);
+}
+
+// eigenvalues (ascending) and eigenvectors (columns of Vec) of a Hermitian
+// n x n matrix; A is overwritten
+void eigh(cvsadc_ctx* c, cplx* A, int n, double* w, cplx* Vec, int max_sweeps) {
+  c->jac.ensure(jacobi_work_bytes(n));
+  jacobi_eigh(c->stream, A, n, w, Vec, max_sweeps, c->jac.p);
 }
 
 void upload(cvsadc_ctx* c, DBuf& dst, const void* src, size_t bytes,
@@ -716,7 +724,7 @@ void build_fns(cvsadc_ctx* c, int prec, double tau) {
   w.ensure(v * sizeof(double) + 64);
   hermitize(c->stream, D.c(), v, v, A.c(), v);
   c->s_small.ensure(4096);
-  jacobi_eigh(c->stream, A.c(), v, w.d(), Vec.c(), 40, c->s_small.d());
+  eigh(c, A.c(), v, w.d(), Vec.c(), 40);
   std::vector<double> occ_asc(v);
   CVS_CUDA(cudaMemcpyAsync(occ_asc.data(), w.p, v * sizeof(double),
                            cudaMemcpyDeviceToHost, c->stream));
@@ -753,7 +761,7 @@ void build_fns(cvsadc_ctx* c, int prec, double tau) {
   Z.ensure((size_t)vk * vk * sizeof(cplx));
   et.ensure(vk * sizeof(double) + 64);
   hermitize(c->stream, Fns.c(), vk, vk, Fh.c(), vk);
-  jacobi_eigh(c->stream, Fh.c(), vk, et.d(), Z.c(), 40, c->s_small.d());
+  eigh(c, Fh.c(), vk, et.d(), Z.c(), 40);
   // U = V~ Z~ (Eq. 20)
   c->fns_U.ensure((size_t)v * vk * sizeof(cplx));
   gemm64(c, v, vk, vk, 1.0, view(Vt.p, vk, 1), view(Z.p, vk, 1),
@@ -1030,13 +1038,6 @@ void build_schur(cvsadc_ctx* c, int prec, double theta, bool cached, bool approx
   }
 }
 
-// scratch of sch_th (doubles): [0,128) per-root theta, [128, 736) partial
-// sums, then the rotation cosines and (16-byte aligned) the sines
-size_t schur_th_doubles(int64_t N1) {
-  const size_t cc_n = (size_t)(N1 / 2 + 2);
-  return 736 + ((cc_n + 1) & ~(size_t)1) + 2 * cc_n;
-}
-
 // Lowest p eigenpairs of the dense Hermitian sch_S (N1 x N1) into sch_U
 // ([N1][p], columns) and sch_lam, by block Davidson with S products as FP64
 // GEMMs, the diagonal preconditioner, FP64 subspace algebra and the Jacobi
@@ -1131,7 +1132,7 @@ void schur_eigh_partial(cvsadc_ctx* c, int p) {
   for (; it < 300; ++it) {
     ts_dot(s, X, m, AX, m, n, tsp, H, m, true);
     hermitize(s, H, m, m, A, m);
-    jacobi_eigh(s, A, m, w, Y, 60, dw);
+    eigh(c, A, m, w, Y, 60);
     const int kk = std::min(p, m);
     // Ritz vectors U = Y[:, :kk]^T X, AU = Y^T AX
     ts_combine(s, X, Y, nullptr, nullptr, m, m, kk, n, U.c(), true);
@@ -1176,10 +1177,6 @@ void schur_eigh_partial(cvsadc_ctx* c, int p) {
 void schur_eigh(cvsadc_ctx* c, bool warm = false) {
   const double t0 = verbose() ? (c->sync(), now_ms()) : 0.0;
   const int64_t N1 = c->N1;
-  const size_t cc_n = (size_t)(N1 / 2 + 2);
-  double* part = c->sch_th.d() + 128;
-  double* cc = c->sch_th.d() + 736;
-  cplx* se = (cplx*)(c->sch_th.d() + 736 + ((cc_n + 1) & ~(size_t)1));
   if (warm) {
     // sch_V = S U_prev; sch_S = U_prev^H sch_V; sch_W keeps U_prev
     c->sch_W.ensure((size_t)N1 * N1 * sizeof(cplx));
@@ -1191,9 +1188,9 @@ void schur_eigh(cvsadc_ctx* c, bool warm = false) {
            conj_of(trans(view(c->sch_W.c(), N1, 1))), view(c->sch_V.c(), N1, 1),
            0.0, view(c->sch_S.c(), N1, 1));
   }
-  const int sweeps =
-      jacobi_eigh_parallel(c->stream, c->sch_S.c(), (int)N1, c->sch_lam.d(),
-                           c->sch_U.c(), c->sch_V.c(), part, cc, se, 30);
+  c->jac.ensure(jacobi_work_bytes((int)N1));
+  const int sweeps = jacobi_eigh_grid(c->stream, c->sch_S.c(), (int)N1, c->sch_lam.d(),
+                                      c->sch_U.c(), c->sch_V.c(), c->jac.p, 30, 1e-10, 1e-7);
   if (warm) {
     // eigenvectors in the original basis: U = U_prev U'
     CVS_CUDA(cudaMemcpyAsync(c->sch_V.p, c->sch_U.p, (size_t)N1 * N1 * sizeof(cplx),
@@ -1274,7 +1271,7 @@ void schur_init(cvsadc_ctx* c) {
   c->sch_C12.ensure((size_t)v * v * nc * nc * sizeof(cplx));
   c->sch_work.ensure((size_t)(2 + nc) * jc * v3 * sizeof(cplx));
   c->sch_tmp.ensure(std::max((size_t)v * v * nc * nc, (size_t)N1 * 64) * sizeof(cplx));
-  c->sch_th.ensure(schur_th_doubles(N1) * sizeof(double) + 256);
+  c->sch_th.ensure(1024 * sizeof(double));  // per-root theta
 }
 
 // Finds theta0 and builds the preconditioner; false when it does not apply
@@ -1517,8 +1514,8 @@ DavResult davidson_impl(cvsadc_ctx* c, int prec, int nroots, int max_iter,
   c->dv_w.ensure((size_t)(msub + 64) * sizeof(double));
   // dv_misc: ts_dot partials [msub*msub*TS_CHUNKS] complex, then a
   // double work area laid out at fixed offsets
-  const size_t W_PART = 0, W_RN2 = 64 * 320, W_JAC = W_RN2 + 128,
-               W_KS = W_JAC + 64, W_IDX = W_KS + 1024, W_NRM = W_IDX + 128,
+  const size_t W_PART = 0, W_RN2 = 64 * 320, W_KS = W_RN2 + 128,
+               W_IDX = W_KS + 1024, W_NRM = W_IDX + 128,
                W_KEPT = W_NRM + 64, W_COEF = W_KEPT + 64,
                W_TOTAL = W_COEF + 2 * (2 * 64 * 64 + 128 * 64);
   c->dv_misc.ensure((size_t)msub * msub * TS_CHUNKS * sizeof(cplx) +
@@ -1630,8 +1627,7 @@ DavResult davidson_impl(cvsadc_ctx* c, int prec, int nroots, int max_iter,
     m_done = m;
     // A = (H + H^H)/2 over m x m (H stored with leading dimension msub)
     hermitize(s, c->dv_H.c(), msub, m, c->dv_A.c(), m);
-    jacobi_eigh(s, c->dv_A.c(), m, c->dv_w.d(), c->dv_U.c(), 60,
-                dwork + W_JAC);
+    eigh(c, c->dv_A.c(), m, c->dv_w.d(), c->dv_U.c(), 60);
     // Ritz vectors and their sigma images for the lowest k
     ts_combine(s, V, c->dv_U.c(), nullptr, nullptr, m, m, k, N, c->dv_X.c(), a64);
     ts_combine(s, nullptr, nullptr, W, c->dv_U.c(), m, m, k, N, c->dv_AX.c(), a64);
@@ -1929,7 +1925,7 @@ FoldResult folded_davidson(cvsadc_ctx* c, int prec, int k, int max_iter, int max
   double* thd = wp + msub;      // [msub]
   double* rn1 = thd + msub;     // [msub]
   double* rnt = rn1 + msub;     // [msub]
-  double* jinfo = rnt + msub;   // jacobi info + misc
+  double* misc = rnt + msub;    // norms and kept counts
   cplx* V = c->fv_V.c();
   cplx* Bo = c->fv_B.c();  // orthonormal basis of span(V) (singles metric)
   cplx* Rf = c->fv_R.c();
@@ -1942,8 +1938,8 @@ FoldResult folded_davidson(cvsadc_ctx* c, int prec, int k, int max_iter, int max
 
   // orthonormal rows of T (cnt) against Bo[0:nb] and within, appended to
   // Bo and (when toV) V; returns how many were kept
-  double* nrm0 = jinfo + 16;
-  int* kept_d = (int*)(jinfo + 16 + 256);
+  double* nrm0 = misc;
+  int* kept_d = (int*)(misc + 256);
   int* src_d = kept_d + 64;
   std::vector<int> src_h(64);
   cplx* G0 = Hp;  // scratch for the block Gram / transform (cnt <= 4k <= msub)
@@ -2066,7 +2062,7 @@ FoldResult folded_davidson(cvsadc_ctx* c, int prec, int k, int max_iter, int max
     // generalised eigenproblem H c = w O c through O^-1/2 (eigenvalues of O
     // below 1e-12 of the largest are dropped)
     hermitize(s, O, msub, m, Hp, m);
-    jacobi_eigh(s, Hp, m, wo, Uo, 60, jinfo);
+    eigh(c, Hp, m, wo, Uo, 60);
     std::vector<double> hw(m);
     CVS_CUDA(cudaMemcpyAsync(hw.data(), wo, m * sizeof(double), cudaMemcpyDeviceToHost, s));
     c->sync();
@@ -2079,7 +2075,7 @@ FoldResult folded_davidson(cvsadc_ctx* c, int prec, int k, int max_iter, int max
     gemm64(c, m, kept, m, 1.0, view(H, msub, 1), view(Oi, m, 1), 0.0, view(Cp, msub, 1));
     gemm64(c, kept, kept, m, 1.0, conj_of(trans(view(Oi, m, 1))), view(Cp, msub, 1), 0.0,
            view(Hp, kept, 1));
-    jacobi_eigh(s, Hp, kept, wp, Yp, 60, jinfo);
+    eigh(c, Hp, kept, wp, Yp, 60);
     const int kk = std::min(k, kept);
     // C = Oi Yp[:, :kk]  ([m][kk], ld msub)
     gemm64(c, m, kk, kept, 1.0, view(Oi, m, 1), view(Yp, kept, 1), 0.0, view(C, msub, 1));
@@ -2835,7 +2831,7 @@ double estimate_bytes(const cvsadc_params* p) {
     const double jc = std::max(1.0, std::min(nw, std::floor(6e9 / per_j)));
     b += z * (nc * v * nc * nw * 2 + nc * nc * v * nw);  // <Kb||Ij>, temps
     b += std::min(nw * v3 * z, 48e9);          // cached <ab||cj>
-    b += 4 * z * N1 * N1 + 8 * N1 + z * nc * v * v + z * v * v * nc * nc;
+    b += 6 * z * N1 * N1 + 12 * N1 + z * nc * v * v + z * v * v * nc * nc;
     b += (2.0 + nc) * jc * v3 * z;             // chunk workspace
     b += z * std::max(v * v * nc * nc, N1 * 64.0) + 8 * (800 + 2 * N1) + 2 * z * N;
   }

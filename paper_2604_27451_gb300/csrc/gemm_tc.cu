@@ -29,7 +29,9 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.cuh"
@@ -557,35 +559,10 @@ void zgemm_tc(cudaStream_t s, int nprod, int M, int N, int K, double alpha,
 // 2^{-7(i+j+2)}, to float-float accumulators (about 48 bits) in registers.
 // The epilogue applies 2^{e_m + f_n}, alpha and beta in FP64.
 //
-// CTA: 576 threads.  Warp 0 lane 0: TMA producer; warp 1 lane 0: MMA
-// issuer; warps 2..17: drain (warp w reads TMEM lanes 32 (w % 4) .. +31 and
-// the 32 columns [32 c, 32 c + 32), c = (w - 2) / 4, of a 128 x 128 tile).
 // ===========================================================================
 namespace {
 
-constexpr int SBN = 128;          // N' per CTA (64 complex columns)
-constexpr int SSTAGES = 7;
-constexpr int S_A_TILE = BM * BK * 2;
-constexpr int S_B_TILE = SBN * BK * 2;
-constexpr int S_STAGE = S_A_TILE + S_B_TILE;
-constexpr int S_SMEM = SSTAGES * S_STAGE + 1024 + 512;
-constexpr int RUN_KT = 16;         // k-tiles per exact run: 16 * 64 = 1024 terms
 constexpr int SLICE_BITS = 7;
-constexpr int MAX_PAIRS = 36;
-
-// Slice pairs (i, j) ordered by order o = i + j, then by i.  With this
-// order the pairs of a 4-slice product (orders 0..3, 10 pairs) are the first
-// 10 of the 7-slice table (orders 0..6, 28 pairs), so one table, fixed at
-// compile time, serves both and no launch ever rewrites constant memory
-// under a kernel running on another stream.
-// slice of A for pair p
-__constant__ int c_si[MAX_PAIRS] = {0, 0, 1, 0, 1, 2, 0, 1, 2, 3,
-                                    0, 1, 2, 3, 4, 0, 1, 2, 3, 4, 5,
-                                    0, 1, 2, 3, 4, 5, 6};
-// slice of B for pair p
-__constant__ int c_sj[MAX_PAIRS] = {0, 1, 0, 2, 1, 0, 3, 2, 1, 0,
-                                    4, 3, 2, 1, 0, 5, 4, 3, 2, 1, 0,
-                                    6, 5, 4, 3, 2, 1, 0};
 
 __device__ __forceinline__ void ff_add(float& hi, float& lo, float x) {
   // TwoSum without contraction
@@ -596,167 +573,474 @@ __device__ __forceinline__ void ff_add(float& hi, float& lo, float x) {
   lo = __fadd_rn(lo, e);
 }
 
-__global__ void __launch_bounds__(576, 1)
-    tc_slice_kernel(const __grid_constant__ CUtensorMap tmA,
-                    const __grid_constant__ CUtensorMap tmB, int npairs,
-                    int ktpp, int kpb, int kb_off, int zl, int M, int N,
-                    const int* __restrict__ eA,
-                    const int* __restrict__ eB, double alpha, double beta,
-                    View C, cplx* part, int* err) {
+// ---------------------------------------------------------------------------
+// The exact-slice GEMM on pairs of CTAs (cta_group::2, NS slices).  Packed
+// operands: A'' row m = 2 NS segments (slice i, re / im) of Kp values, B''
+// rows 2n (the real output column) and 2n + 1 (the imaginary one) = 2 NS
+// segments (slice j, re-part / im-part: [re b, -im b] for row 2n and
+// [im b, re b] for row 2n + 1).  One unit is one K block of 64 in one part:
+// the NS tiles of A (128 rows in each CTA) and of B, from which all the NS
+// (NS + 1) / 2 slice pairs are issued.  Pairs of one order o = i + j share
+// the scale 2^{-7(o+2)} and one tensor-memory accumulator of PN columns; the
+// orders lie side by side and fill the tensor memory (4 x 128, or 7 x 64 and
+// 64 that nothing reads), so there is one set of them.
+//
+// Exact runs: |q_0| <= 2^7, |q_i| <= 2^6 for i > 0, so a run of 512 products
+// (8 units) of every pair of an order stays within 2^23 (o = 0, 1), 2.5 2^22
+// (o = 2), 3 2^22 (o = 3), 3.5 2^22 (o = 4) and 2^24 (o = 5) and sums exactly
+// in FP32; order 6 may pass 2^24 by an eighth, where one rounding is 2^-55 of
+// the order-0 product it is added to.  At the end of a run the orders finish
+// one after the other, the drain warps add each to float-float accumulators
+// in registers, and the next run overwrites an order once it is in registers.
+//
+// What bounds it: an MMA takes 90 to 100 cycles to issue and run whatever its
+// width up to 128 columns, and a unit's operands arrive at ~11 TB/s over all
+// SMs (96 KB a unit and CTA: 1.35 us).
+// - 4 slices: a B slice is split over the CTAs by columns, 40 MMAs of 256 x
+//   128 a unit.  One thread issues an MMA in 45 ns or more, so two warps do,
+//   each with its own orders: 2.1 -> 1.8 us a unit.
+// - 7 slices: the 112 MMAs of 256 x 64 took 5.0 us a unit however many warps
+//   issued them.  B slices are whole in one CTA instead, so that one MMA
+//   covers up to four (256 columns: two slices from either CTA, into four
+//   adjacent orders): 44 MMAs, 2.75 us a unit.
+// A's tiles free up one by one, so the copies run more than a unit ahead.
+// The pairs of CTAs are persistent: the epilogue of a tile runs while the
+// next one's first run is computed.  Measured (with the operands packed):
+// 4096^3 4 slices 4.57 -> 3.23 ms (170 TFLOP/s, 0.91 of the measured bf16
+// rate over 10 products; the tile kernel below before), 7 slices 21.2 -> 9.5
+// ms (58 TFLOP/s, 0.87 over 28 products).
+//
+// Warps: 0 (lane 0) TMA producer; 1 .. ISSUERS of rank 0 (lane 0) MMA
+// issuers; then 16 drain warps (warp w reads TMEM lanes 32 (w % 4) .. +31
+// and CG columns of every order).  CTA rank r owns rows 128 r .. of the tile.
+// ---------------------------------------------------------------------------
+template <int NS>
+struct PairCfg;
+template <>
+struct PairCfg<4> {
+  static constexpr int PN = 128, ASLOTS = 8, BSTAGES = 3, ISSUERS = 2;
+  static constexpr int R0 = 0, R1 = 0, R2 = 0, R3 = 0;
+  static constexpr int B_ROWS = 4 * PN / 2;  // half of every slice
+};
+template <>
+struct PairCfg<7> {
+  static constexpr int PN = 64, ASLOTS = 9, BSTAGES = 2, ISSUERS = 1;
+  // rows of the B regions of a stage: B_0 .. B_3 (two slices in each CTA),
+  // B_4 | B_5, B_0 | B_1 (one in each), B_6 (half in each)
+  static constexpr int R0 = 0, R1 = 128, R2 = 192, R3 = 256, B_ROWS = 288;
+};
+constexpr int P_BM = 256;
+constexpr int P_RUN = 8;  // units per exact run
+template <int NS>
+constexpr int pair_threads() {
+  return 32 * (1 + PairCfg<NS>::ISSUERS + 16);
+}
+template <int NS>
+constexpr int pair_smem() {
+  using P = PairCfg<NS>;
+  return P::ASLOTS * A_TILE + P::BSTAGES * P::B_ROWS * BK * 2 + 1024 + 512;
+}
+
+__device__ __forceinline__ uint32_t cta_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// the shared::cluster address of `p`'s counterpart in CTA 0 of the pair
+__device__ __forceinline__ uint32_t leader_addr(const void* p) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(smem_u32(p)));
+  return a;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile(
+      "barrier.cluster.arrive.release.aligned;\n"
+      "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// copy into this CTA's shared memory, counted on the leader's barrier
+__device__ __forceinline__ void tma_load2(const CUtensorMap* map, uint32_t leader_bar,
+                                          void* dst, int x, int y) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::"
+      "bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(smem_u32(dst)),
+      "l"((uint64_t)map), "r"(leader_bar), "r"(x), "r"(y)
+      : "memory");
+}
+// 2^e for the exponents of a line (-1022 .. 1025; infinite above 1023)
+__device__ __forceinline__ double pow2(int e) {
+  return __hiloint2double(min(2047, 1023 + e) << 20, 0);
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+  uint32_t r[8];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7])
+      : "r"(taddr)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void umma2(uint32_t dtm, uint64_t a, uint64_t b, uint32_t idesc,
+                                      uint32_t acc) {
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(dtm),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc));
+}
+// arrives on the barrier's counterparts in both CTAs once this thread's MMAs
+// issued so far are done
+__device__ __forceinline__ void umma2_commit(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster"
+      ".b64 [%0], %1;" ::"r"(smem_u32(bar)),
+      "h"((uint16_t)3)
+      : "memory");
+}
+
+template <int NS>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 1)
+    tc_slice_pair_kernel(const __grid_constant__ CUtensorMap tmA,
+                         const __grid_constant__ CUtensorMap tmB,
+                         const __grid_constant__ CUtensorMap tmB2, int kpa, int ka_off,
+                         int kpb, int kb_off, int nkb, int zl, int ntm, int ntn, int nitems,
+                         int M, int N, const int* __restrict__ eA, const int* __restrict__ eB,
+                         double alpha, double beta, View C, cplx* part, int* err) {
+  using P = PairCfg<NS>;
+  constexpr int PN = P::PN, AS = P::ASLOTS, BS = P::BSTAGES, NI = P::ISSUERS;
+  constexpr int CG = PN / 4;                       // columns of an order per drain warp
+  constexpr int B_SLICE = (PN / 2) * BK * 2;       // this CTA's half of a B slice tile
+  constexpr int B_STAGE = P::B_ROWS * BK * 2;
+  constexpr uint32_t TMEM_COLS = 512;
+  static_assert(NS * PN <= (int)TMEM_COLS, "accumulators fit the tensor memory");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sA = smem;
-  uint8_t* sB = smem + SSTAGES * S_A_TILE;
-  uint64_t* full = (uint64_t*)(smem + SSTAGES * S_STAGE);
-  uint64_t* empty = full + SSTAGES;
-  uint64_t* afull = empty + SSTAGES;  // [2]
-  uint64_t* aempty = afull + 2;       // [2]
-  uint32_t* tslot = (uint32_t*)(aempty + 2);
+  uint8_t* sB = smem + AS * A_TILE;
+  uint64_t* fullA = (uint64_t*)(sB + BS * B_STAGE);
+  uint64_t* emptyA = fullA + AS;
+  uint64_t* fullB = emptyA + AS;
+  uint64_t* emptyB = fullB + BS;
+  uint64_t* afull = emptyB + BS;   // [NS]
+  uint64_t* aempty = afull + NS;   // [NS]
+  uint32_t* tslot = (uint32_t*)(aempty + NS);
   __shared__ int fail;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int mt, nt;
-  tile_coords(mt, nt);
-  const int m0 = mt * BM, n0 = nt * SBN;
-  const int z = blockIdx.z;
-  // this CTA's k-tiles of every pair: [zb, ze) relative to the pair start
-  const int zb = z * zl, ze = min(ktpp, zb + zl);
-  const int zlen = max(0, ze - zb);
-  const int runs_pp = (zlen + RUN_KT - 1) / RUN_KT;
-  const int nruns = npairs * runs_pp;
+  const uint32_t rank = cta_rank();
+  const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
 
   if (threadIdx.x == 0) {
     fail = 0;
-    for (int s = 0; s < SSTAGES; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+    for (int s = 0; s < AS; ++s) {
+      mbar_init(&fullA[s], 1);
+      mbar_init(&emptyA[s], NI);
     }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&afull[b], 1);
-      mbar_init(&aempty[b], 16);
+    for (int s = 0; s < BS; ++s) {
+      mbar_init(&fullB[s], 1);
+      mbar_init(&emptyB[s], NI);
+    }
+    for (int o = 0; o < NS; ++o) {
+      mbar_init(&afull[o], 1);
+      mbar_init(&aempty[o], 32);  // the drain warps of both CTAs
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncwarp();
   if (warp == 0) {
     asm volatile(
-        "tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+        "tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
             smem_u32(tslot)),
-        "r"(2 * SBN));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        "r"(TMEM_COLS));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
   }
   fence_before();
   __syncthreads();
+  cluster_sync();
   fence_after();
   const uint32_t tmem = *tslot;
 
+  // item -> first row and column of its tile, its K blocks [kb0, kb1)
+  auto item_at = [&](int it, int& m0, int& n0, int& z, int& kb0, int& kb1) {
+    const int tiles = ntm * ntn;
+    z = it / tiles;
+    const int t = it - z * tiles;
+    // groups of 4 M tiles walked column by column (shared panels in L2)
+    const int per_group = 4 * ntn;
+    const int g = t / per_group, first = 4 * g;
+    const int gsz = min(ntm - first, 4);
+    const int local = t - g * per_group;
+    m0 = (first + local % gsz) * P_BM;
+    n0 = (local / gsz) * (PN / 2);  // complex columns
+    kb0 = z * zl;
+    kb1 = min(nkb, kb0 + zl);
+  };
+
   if (threadIdx.x == 0) {
-    // TMA producer over this CTA's k-tiles of every pair
-    const int nkt = npairs * zlen;
-    for (int i = 0; i < nkt; ++i) {
-      const int p = i / zlen, t = zb + i % zlen;  // pair, k-tile within it
-      const int kt = p * ktpp + t;
-      // B: segment 2 p + (re / im half), K block kb_off + (t mod Kp / BK)
-      const int hk = ktpp >> 1;
-      const int xb = (2 * p + t / hk) * kpb + (kb_off + t % hk) * BK;
-      const int s = i % SSTAGES;
-      const uint32_t ph = (i / SSTAGES) & 1;
-      if (i >= SSTAGES && !mbar_wait(&empty[s], ph ^ 1)) {
-        fail = 1;
-        break;
-      }
-      if (fail) break;
-      mbar_expect_tx(&full[s], S_STAGE);
-      tma_load(&tmA, &full[s], sA + s * S_A_TILE, kt * BK, m0);
-      tma_load(&tmB, &full[s], sB + s * S_B_TILE, xb, n0);
-    }
-  } else if (threadIdx.x == 32) {
-    // MMA issuer: one exact run per (pair, run) into alternating buffers
-    const uint32_t id = idesc_bf16(BM, SBN);
-    int i = 0;  // position in the producer's sequence
-    for (int r = 0; r < nruns && !fail; ++r) {
-      const int rr = r % runs_pp;
-      const int i0 = i, i1 = i + min(RUN_KT, zlen - rr * RUN_KT);
-      const int b = r & 1;
-      if (r >= 2 && !mbar_wait(&aempty[b], ((r >> 1) + 1) & 1)) {
-        fail = 4;
-        break;
-      }
-      fence_after();
-      const uint32_t dt = tmem + (uint32_t)(b * SBN);
-      for (i = i0; i < i1; ++i) {
-        const int s = i % SSTAGES;
-        const uint32_t ph = (i / SSTAGES) & 1;
-        if (!mbar_wait(&full[s], ph)) {
-          fail = 2;
+    // TMA producer of this CTA's rows of A and half of the columns of B
+    int u = 0, ia = 0;  // units and A tiles so far
+    for (int it = pair; it < nitems && !fail; it += npairs) {
+      int m0, n0, z, kb0, kb1;
+      item_at(it, m0, n0, z, kb0, kb1);
+      const int ya = m0 + (int)rank * BM, yb = 2 * n0 + (int)rank * (PN / 2);
+      for (int v = 0; v < 2 * (kb1 - kb0) && !fail; ++v, ++u) {
+        const int kb = kb0 + v / 2, c = v & 1;
+        const int sb = u % BS;
+        if (u >= BS && !mbar_wait(&emptyB[sb], ((u / BS) & 1) ^ 1)) {
+          fail = 1;
           break;
         }
-        fence_after();
-        const uint64_t ad = sdesc(smem_u32(sA + s * S_A_TILE));
-        const uint64_t bd = sdesc(smem_u32(sB + s * S_B_TILE));
+        if (rank == 0) mbar_expect_tx(&fullB[sb], 2 * B_STAGE);
+        const uint32_t fb = leader_addr(&fullB[sb]);
+        uint8_t* st = sB + sb * B_STAGE;
+        const int xb = c * kpb + (kb_off + kb) * BK;  // slice j: + 2 j kpb
+        if constexpr (NS == 4) {
 #pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk)
-          umma(dt, ad + 2 * kk, bd + 2 * kk, id, (i != i0 || kk) ? 1u : 0u);
-        umma_commit(&empty[s]);
+          for (int j = 0; j < NS; ++j)
+            tma_load2(&tmB, fb, st + j * B_SLICE, 2 * j * kpb + xb, yb);
+        } else {
+          auto slice = [&](int row, int j) {  // all 64 columns of slice j
+            tma_load2(&tmB, fb, st + row * BK * 2, 2 * j * kpb + xb, 2 * n0);
+          };
+          slice(P::R0, rank ? 2 : 0);
+          slice(P::R0 + PN, rank ? 3 : 1);
+          slice(P::R1, rank ? 5 : 4);
+          slice(P::R2, rank ? 1 : 0);
+          tma_load2(&tmB2, fb, st + P::R3 * BK * 2, 2 * 6 * kpb + xb, yb);
+        }
+        for (int i = 0; i < NS; ++i, ++ia) {
+          const int sa = ia % AS;
+          if (ia >= AS && !mbar_wait(&emptyA[sa], ((ia / AS) & 1) ^ 1)) {
+            fail = 1;
+            break;
+          }
+          if (rank == 0) mbar_expect_tx(&fullA[sa], 2 * A_TILE);
+          tma_load2(&tmA, leader_addr(&fullA[sa]), sA + sa * A_TILE,
+                    (2 * i + c) * kpa + (ka_off + kb) * BK, ya);
+        }
       }
-      umma_commit(&afull[b]);
     }
-  } else if (warp >= 2) {
-    // drain warps
-    const int q = warp & 3;            // TMEM lane quarter
-    const int cq = (warp - 2) >> 2;     // 32-column quarter of the tile
-    float hi[32], lo[32];
+  } else if (warp >= 1 && warp <= NI) {
+    if (rank == 0 && lane == 0) {
+      const uint32_t dhi = (uint32_t)(sdesc(0) >> 32);
+      auto desc = [&](uint32_t lo) { return ((uint64_t)dhi << 32) | lo; };
+      // NS = 4: issuer w takes the orders 3 - w and w, five pairs a step
+      [[maybe_unused]] auto issue4 = [&](auto W) {
+        constexpr int w = decltype(W)::value;
+        constexpr int O1 = NS - 1 - w, O2 = w;
+        const uint32_t id = idesc_bf16(P_BM, PN);
+        int u = 0, ia = 0, r = 0;
+        for (int it = pair; it < nitems && !fail; it += npairs) {
+          int m0, n0, z, kb0, kb1;
+          item_at(it, m0, n0, z, kb0, kb1);
+          const int nu = 2 * (kb1 - kb0);
+          for (int v = 0; v < nu && !fail; ++v, ++u) {
+            const bool first = v % P_RUN == 0;
+            const bool last = v % P_RUN == P_RUN - 1 || v == nu - 1;
+            const int sb = u % BS;
+            bool ok = mbar_wait(&fullB[sb], (u / BS) & 1);
+            // low words of the descriptors (the high word is the same for all)
+            const uint32_t bd = (uint32_t)sdesc(smem_u32(sB + sb * B_STAGE));
+            // pair (i, o - i) into order o
+            auto mma = [&](int i, int o, uint32_t ad, bool start) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) hi[i] = lo[i] = 0.f;
+              for (int kk = 0; kk < BK / 16; ++kk)
+                umma2(tmem + o * PN, desc(ad + 2 * kk),
+                      desc(bd + (o - i) * (B_SLICE >> 4) + 2 * kk), id,
+                      (start && kk == 0) ? 0u : 1u);
+            };
+            if (first || last) {
+              // by order: it waits for its drain at the start of a run and is
+              // handed to the drain warps at the end
+              uint32_t ad[NS];
+#pragma unroll
+              for (int i = 0; i < NS; ++i) {
+                const int sa = (ia + i) % AS;
+                ok = ok && mbar_wait(&fullA[sa], ((ia + i) / AS) & 1);
+                ad[i] = (uint32_t)sdesc(smem_u32(sA + sa * A_TILE));
+              }
+#pragma unroll
+              for (int o = 0; o < NS; ++o) {
+                if (o != O1 && o != O2) continue;
+                if (first && r > 0) ok = ok && mbar_wait(&aempty[o], (r - 1) & 1);
+                if (!ok) break;
+                fence_after();
+#pragma unroll
+                for (int i = 0; i <= o; ++i) mma(i, o, ad[i], first && i == 0);
+                if (last) umma2_commit(&afull[o]);
+              }
+              if (ok)
+#pragma unroll
+                for (int i = 0; i < NS; ++i) umma2_commit(&emptyA[(ia + i) % AS]);
+            } else {
+              // by slice of A, whose slot is freed early
+#pragma unroll
+              for (int i = 0; i < NS; ++i) {
+                const int sa = (ia + i) % AS;
+                // also where no pair needs A_i: its slot is not given back
+                // before it has been filled
+                ok = ok && mbar_wait(&fullA[sa], ((ia + i) / AS) & 1);
+                if (!ok) break;
+                fence_after();
+                const uint32_t ad = (uint32_t)sdesc(smem_u32(sA + sa * A_TILE));
+                if (O1 >= i) mma(i, O1, ad, false);
+                if (O2 >= i) mma(i, O2, ad, false);
+                umma2_commit(&emptyA[sa]);
+              }
+            }
+            if (!ok) {
+              fail = 2;
+              break;
+            }
+            umma2_commit(&emptyB[sb]);
+            ia += NS;
+            if (last) ++r;
+          }
+        }
+      };
+      // NS = 7: one issuer, up to four slices of B per MMA
+      [[maybe_unused]] auto issue7 = [&]() {
+        int u = 0, ia = 0, r = 0;
+        for (int it = pair; it < nitems && !fail; it += npairs) {
+          int m0, n0, z, kb0, kb1;
+          item_at(it, m0, n0, z, kb0, kb1);
+          const int nu = 2 * (kb1 - kb0);
+          for (int v = 0; v < nu && !fail; ++v, ++u) {
+            const bool first = v % P_RUN == 0;
+            const bool last = v % P_RUN == P_RUN - 1 || v == nu - 1;
+            const int sb = u % BS;
+            bool ok = mbar_wait(&fullB[sb], (u / BS) & 1);
+            const uint32_t bd = (uint32_t)sdesc(smem_u32(sB + sb * B_STAGE));
+            // A_i with the slices of the region at `row` into orders o ..
+            auto mma = [&](int o, uint32_t ad, int row, int n, bool start) {
+              const uint32_t id = idesc_bf16(P_BM, n);
+#pragma unroll
+              for (int kk = 0; kk < BK / 16; ++kk)
+                umma2(tmem + o * PN, desc(ad + 2 * kk),
+                      desc(bd + row * (BK * 2 >> 4) + 2 * kk), id, (start && kk == 0) ? 0u : 1u);
+            };
+            // the drains of orders [o0, o1) at the start of a run
+            auto drained = [&](int o0, int o1) {
+              for (int o = o0; o < o1 && first && r > 0; ++o)
+                ok = ok && mbar_wait(&aempty[o], (r - 1) & 1);
+              if (ok) fence_after();
+              return ok;
+            };
+#pragma unroll
+            for (int i = 0; i < NS; ++i) {
+              const int sa = (ia + i) % AS;
+              ok = ok && mbar_wait(&fullA[sa], ((ia + i) / AS) & 1);
+              if (!ok) break;
+              fence_after();
+              const uint32_t ad = (uint32_t)sdesc(smem_u32(sA + sa * A_TILE));
+              if (i < 5) {
+                if (i == 0 && !drained(0, 4)) break;
+                mma(i, ad, P::R0, 4 * PN, first && i == 0);
+              }
+              if (i < 3) {
+                if (i == 0 && !drained(4, 6)) break;
+                mma(i + 4, ad, P::R1, 2 * PN, first && i == 0);
+              }
+              if (i == 0) {
+                if (!drained(6, 7)) break;
+                mma(6, ad, P::R3, PN, first);
+              }
+              if (i >= 5) mma(i, ad, P::R2, 2 * PN, false);
+              umma2_commit(&emptyA[sa]);
+              // no later pair of this unit adds to order i
+              if (last) umma2_commit(&afull[i]);
+            }
+            if (!ok) {
+              fail = 2;
+              break;
+            }
+            umma2_commit(&emptyB[sb]);
+            ia += NS;
+            if (last) ++r;
+          }
+        }
+      };
+      if constexpr (NS == 4) {
+        if (warp == 1) issue4(std::integral_constant<int, 0>());
+        if (warp == 2) issue4(std::integral_constant<int, 1>());
+      } else {
+        issue7();
+      }
+    }
+  } else if (warp > NI) {
+    // drain warps
+    const int q = warp & 3;               // TMEM lane quarter
+    const int cq = (warp - 1 - NI) >> 2;  // CG columns of every order
+    const uint32_t ae = leader_addr(aempty);
     bool ok = true;
-    for (int r = 0; r < nruns; ++r) {
-      const int p = r / runs_pp;
-      const int b = r & 1;
-      if (!mbar_wait(&afull[b], (r >> 1) & 1)) {
+    int r = 0;
+    for (int it = pair; it < nitems && ok; it += npairs) {
+      int m0, n0, z, kb0, kb1;
+      item_at(it, m0, n0, z, kb0, kb1);
+      const int nruns = (2 * (kb1 - kb0) + P_RUN - 1) / P_RUN;
+      float hi[CG], lo[CG];
+#pragma unroll
+      for (int i = 0; i < CG; ++i) hi[i] = lo[i] = 0.f;
+      for (int rr = 0; rr < nruns && ok; ++rr, ++r) {
+#pragma unroll 1
+        for (int o = 0; o < NS; ++o) {
+          if (!mbar_wait(&afull[o], r & 1)) {
+            ok = false;
+            break;
+          }
+          fence_after();
+          // 2^{-7 (o + 2)}
+          const float sc = __int_as_float((127 - SLICE_BITS * (o + 2)) << 23);
+#pragma unroll
+          for (int h = 0; h < CG / 8; ++h) {
+            float v[8];
+            tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(o * PN + cq * CG + 8 * h), v);
+            if (h == CG / 8 - 1) {
+              // the order is in registers: the next run may overwrite it
+              fence_before();
+              __syncwarp();
+              if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(
+                                 ae + 8 * o)
+                             : "memory");
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              ff_add(hi[8 * h + i], lo[8 * h + i], v[i] * sc);
+              // one group of 8 at a time: the accumulators take most registers
+              asm volatile("" : "+f"(hi[8 * h + i]), "+f"(lo[8 * h + i]));
+            }
+          }
+        }
+      }
+      if (!ok || fail) {
         ok = false;
+        if (lane == 0) atomicExch(err, fail ? fail : 3);
         break;
       }
-      fence_after();
-      const float sc = exp2f(-(float)(SLICE_BITS * (c_si[p] + c_sj[p] + 2)));
-      const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) +
-                            (uint32_t)(b * SBN + cq * 32);
-#pragma unroll
-      for (int c2 = 0; c2 < 2; ++c2) {
-        float v[16];
-        tmem_ld16(base + 16 * c2, v);
-#pragma unroll
-        for (int i = 0; i < 16; ++i)
-          ff_add(hi[16 * c2 + i], lo[16 * c2 + i], v[i] * sc);
-      }
-      fence_before();
-      __syncwarp();
-      if (lane == 0) {
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(
-                         smem_u32(&aempty[b]))
-                     : "memory");
-      }
-    }
-    if (!ok || fail) {
-      if (lane == 0) atomicExch(err, fail ? fail : 3);
-    } else {
-      const int m = m0 + q * 32 + lane;
+      const int m = m0 + (int)rank * BM + q * 32 + lane;
       if (m < M) {
         const int64_t ro = part ? 0 : vrow(C, m);
-        const double em = ldexp(1.0, eA[m]);
+        const double em = alpha * pow2(eA[m]);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int n = (n0 + cq * 32) / 2 + i;
+        for (int i = 0; i < CG / 2; ++i) {
+          const int n = n0 + cq * (CG / 2) + i;
           if (n < N) {
-            const double s = alpha * em * ldexp(1.0, eB[n]);
-            cplx o = cmake(s * ((double)hi[2 * i] + (double)lo[2 * i]),
-                           s * ((double)hi[2 * i + 1] + (double)lo[2 * i + 1]));
+            // one column at a time (nothing hoisted): the accumulators take
+            // most registers
+            asm volatile("" : "+f"(hi[2 * i]), "+f"(lo[2 * i]), "+f"(hi[2 * i + 1]),
+                         "+f"(lo[2 * i + 1]) :: "memory");
+            const double sc = em * pow2(eB[n]);
+            cplx o = cmake(sc * ((double)hi[2 * i] + (double)lo[2 * i]),
+                           sc * ((double)hi[2 * i + 1] + (double)lo[2 * i + 1]));
             if (part) {
               part[((int64_t)z * M + m) * N + n] = o;
               continue;
             }
             cplx* d = C.p + ro + vcol(C, n);
             if (beta != 0.0) {
-              cplx old = *d;
+              const cplx old = *d;
               o.x += beta * old.x;
               o.y += beta * old.y;
             }
@@ -766,12 +1050,20 @@ __global__ void __launch_bounds__(576, 1)
       }
     }
   }
+  __syncwarp();
+  // an expired wait: let the copies in flight land before the memory goes
+  if (threadIdx.x == 0 && fail) {
+    const uint64_t t0 = gtime();
+    for (int n = 0; n < (1 << 20) && gtime() - t0 < 2000000; ++n) __nanosleep(1000);
+  }
+  if (threadIdx.x == 0 && fail) atomicExch(err, fail);
   fence_before();
   __syncthreads();
+  __syncwarp();
+  cluster_sync();
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(
-                     tmem),
-                 "r"(2 * SBN));
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"(TMEM_COLS));
 }
 
 // Exponents and slices work on the IEEE bits with integer arithmetic (this
@@ -790,52 +1082,45 @@ __device__ __forceinline__ int64_t vcol32(const View& v, int c) {
   return (int64_t)h * v.cs_hi + (int64_t)(c - h * v.c_lo) * v.cs_lo;
 }
 
-// Exponents over [k0, k0 + K): e with max |re|, |im| < 2^e for every
-// element of a row of A (row_exp) or a column of B (col_exp); an all-zero
-// line gets -1022.  A warp takes one (line, K segment of EXP_SEG) task and
-// folds its maximum into e[] with atomicMax, so an operand with few lines
-// and a K in the millions still spreads over every SM; the caller presets
-// e[] below -1022 (bytes 0x80).
-constexpr int EXP_SEG = 4096;
-__global__ void row_exp_kernel(View A, int M, int K, int k0, int* e) {
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int nsg = (K + EXP_SEG - 1) / EXP_SEG;
-  const int64_t ntask = (int64_t)M * nsg;
-  for (int64_t t = warp; t < ntask; t += nwarp) {
-    const int m = (int)(t / nsg), k1 = (int)(t % nsg) * EXP_SEG;
-    const int k2 = min(K, k1 + EXP_SEG);
-    const int64_t ro = vrow(A, m);
-    int mx = 0;
-    for (int k = k1 + lane; k < k2; k += 32) {
-      const cplx a = A.p[ro + vcol32(A, k0 + k)];
-      mx = max(mx, max(exp_field(a.x), exp_field(a.y)));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) atomicMax(e + m, mx - 1022);
-  }
-}
+// Operands are packed line by line: rows of A, columns of B (a transposed
+// view), so that lines are the view's rows and k its columns.
 
-__global__ void col_exp_kernel(View B, int K, int k0, int N, int* e) {
+// Exponents over [k0, k0 + K): e with max |re|, |im| < 2^e for every element
+// of a line; an all-zero line gets -1022.  The caller presets e[] below
+// -1022 (bytes 0x80); maxima are folded into it with atomicMax, so that an
+// operand with few lines and a K in the millions still spreads over every
+// SM.  KFAST: a warp takes a (line, segment of EXP_SEG) task, lanes along k.
+// Otherwise (the lines are the contiguous mode: columns of a row-major B,
+// (a, b) rows of B^P) lanes take adjacent lines and walk a segment, so that
+// the warp reads 512 contiguous bytes a step instead of half a sector each.
+constexpr int EXP_SEG = 4096, EXP_SEG_LINES = 64;
+template <bool KFAST>
+__global__ void __launch_bounds__(256) line_exp_kernel(View X, int L, int K, int k0, int* e) {
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int nsg = (K + EXP_SEG - 1) / EXP_SEG;
-  const int64_t ntask = (int64_t)N * nsg;
-  for (int64_t t = warp; t < ntask; t += nwarp) {
-    const int n = (int)(t / nsg), k1 = (int)(t % nsg) * EXP_SEG;
-    const int k2 = min(K, k1 + EXP_SEG);
-    const int64_t co = vcol(B, n);
+  constexpr int SEG = KFAST ? EXP_SEG : EXP_SEG_LINES;
+  const int nsg = (K + SEG - 1) / SEG;
+  const int64_t nlg = KFAST ? L : (L + 31) / 32;  // lines, or groups of 32
+  for (int64_t t = warp; t < nlg * nsg; t += nwarp) {
+    const int64_t lg = t / nsg;
+    const int k1 = (int)(t % nsg) * SEG, k2 = min(K, k1 + SEG);
+    const int l = (int)(KFAST ? lg : lg * 32 + lane);
     int mx = 0;
-    for (int k = k1 + lane; k < k2; k += 32) {
-      const cplx b = B.p[vrow(B, k0 + k) + co];
-      mx = max(mx, max(exp_field(b.x), exp_field(b.y)));
+    if (l < L) {
+      const cplx* x = X.p + vrow(X, l);
+      for (int k = KFAST ? k1 + lane : k1; k < k2; k += KFAST ? 32 : 1) {
+        const cplx a = x[vcol32(X, k0 + k)];
+        mx = max(mx, max(exp_field(a.x), exp_field(a.y)));
+      }
     }
+    if (KFAST) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) atomicMax(e + n, mx - 1022);
+      for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      if (lane == 0) atomicMax(e + l, mx - 1022);
+    } else if (l < L) {
+      atomicMax(e + l, mx - 1022);
+    }
   }
 }
 
@@ -844,116 +1129,173 @@ unsigned warp_tasks_grid(int64_t lines, int K, int seg) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>((ntask + 7) / 8, 152 * 32));
 }
 
-// S balanced 7-bit slices of t = x 2^-e (|t| < 1): T = round(t 2^(7S))
-// in integer arithmetic, then digits q_{S-1} .. q_1 in [-64, 63] from the
-// bottom and q_0 = the rest, in [-128, 128], so that
-// t = sum_i q_i 2^(-7(i+1)) + r with |r| <= 2^(-7S-1); each q_i is exact
-// in bf16.
+// S balanced 7-bit slices of t = x 2^-e (|t| < 1): T = round(t 2^(7S)),
+// then digits q_{S-1} .. q_1 in [-64, 63] from the bottom and q_0 = the
+// rest, in [-128, 128], so that t = sum_i q_i 2^(-7(i+1)) + r with |r| <=
+// 2^(-7S-1); each q_i is exact in bf16, the upper half of its float.
+//
+// In 32-bit integer arithmetic: with s = 1075 + e - 7S - E >= 53 - 7S
+// the bits to drop, T = ((m >> (s - 1)) + 1) >> 1.  Adding 64 at every lower
+// digit's place makes its balanced digit the plain one less 64, and a digit
+// n becomes the float n - 64 by an OR into the mantissa of 1.5 2^23 and a
+// subtraction.  (64-bit digits and int-to-float conversions held the packing
+// kernels to 2 TB/s.)
+__device__ __forceinline__ float digit(int n) {  // n in [0, 127]: n - 64
+  return __int_as_float(0x4B400000 | n) - 12582976.0f;
+}
 template <int S>
-__device__ __forceinline__ void slices(double x, int e, __nv_bfloat16* q) {
-  const long long bits = __double_as_longlong(x);
-  const int E = (int)((bits >> 52) & 0x7FF);
-  long long T = 0;
-  if (E != 0) {
-    const long long m = (bits & 0xFFFFFFFFFFFFFLL) | (1LL << 52);
-    const int sh = E - 1075 - e + SLICE_BITS * S;
-    if (sh >= 0)
-      T = m << sh;
-    else if (sh > -63)
-      T = (m + (1LL << (-sh - 1))) >> (-sh);
-    if (bits < 0) T = -T;
+__device__ __forceinline__ void slices(double x, int e, float* q) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const int E = (hi >> 20) & 0x7FF;
+  const uint32_t mh = (hi & 0xFFFFF) | 0x100000;
+  const int s = 1075 + e - 7 * S - E;  // >= 53 - 7 S, since |x| < 2^e
+  if constexpr (S == 4) {
+    const int h = (int)__funnelshift_l(lo, mh, 8);  // m >> 24
+    int T = ((h >> min(31, max(0, s - 25))) + 1) >> 1;
+    T = E == 0 ? 0 : ((int)hi < 0 ? -T : T);
+    T += 64 + (64 << 7) + (64 << 14);
+    q[3] = digit(T & 127);
+    q[2] = digit((T >> 7) & 127);
+    q[1] = digit((T >> 14) & 127);
+    q[0] = __int_as_float(0x4B400000 + (T >> 21)) - 12582912.0f;
+  } else {
+    static_assert(S == 7, "4 or 7 slices");
+    const long long m = ((long long)mh << 32) | lo;
+    long long T = ((m >> min(63, max(0, s - 1))) + 1) >> 1;
+    T = E == 0 ? 0 : ((int)hi < 0 ? -T : T);
+    // 64 at the places of digits 6 .. 1
+    T += 64ll * (1 + (1ll << 7) + (1ll << 14) + (1ll << 21) + (1ll << 28) + (1ll << 35));
+    const int tl = (int)(T & 0xFFFFFFF), th = (int)(T >> 28);
+    q[6] = digit(tl & 127);
+    q[5] = digit((tl >> 7) & 127);
+    q[4] = digit((tl >> 14) & 127);
+    q[3] = digit((tl >> 21) & 127);
+    q[2] = digit(th & 127);
+    q[1] = digit((th >> 7) & 127);
+    q[0] = __int_as_float(0x4B400000 + (th >> 14)) - 12582912.0f;
   }
+}
+// two exact bf16 values as one word
+__device__ __forceinline__ uint32_t bf16_pair(float a, float b) {
+  return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+}
+
+// Packed lines: out line l (A: one, B: the two lines 2l and 2l + 1) = 2 S
+// segments of Kp, segment 2 i + {0: re, 1: im} of slice i; for B line 2l
+// holds [re, -im] and line 2l + 1 [im, re].  Two adjacent k per lane.
+template <int S, bool ISB>
+__device__ __forceinline__ void pack_two(cplx a0, cplx a1, int e, __nv_bfloat16* o, int64_t ld,
+                                         int Kp) {
+  float r0[S], i0[S], r1[S], i1[S];
+  slices<S>(a0.x, e, r0);
+  slices<S>(a0.y, e, i0);
+  slices<S>(a1.x, e, r1);
+  slices<S>(a1.y, e, i1);
 #pragma unroll
-  for (int i = S - 1; i > 0; --i) {
-    const long long d = ((T + 64) & 127) - 64;
-    q[i] = __float2bfloat16_rn((float)d);
-    T = (T - d) >> SLICE_BITS;
+  for (int i = 0; i < S; ++i) {
+    const uint32_t re = bf16_pair(r0[i], r1[i]), im = bf16_pair(i0[i], i1[i]);
+    __nv_bfloat16* p = o + (2 * i) * (int64_t)Kp;
+    *(uint32_t*)p = re;
+    if (!ISB) {
+      *(uint32_t*)(p + Kp) = im;
+    } else {
+      *(uint32_t*)(p + Kp) = bf16_pair(-i0[i], -i1[i]);
+      *(uint32_t*)(p + ld) = im;
+      *(uint32_t*)(p + ld + Kp) = re;
+    }
   }
-  q[0] = __float2bfloat16_rn((float)T);
 }
 
-// A' [Mp][2 npairs Kp]: row m, segment 2p + {0: re, 1: im} of slice c_si[p].
-// A warp takes one (row, K segment of PACK_SEG) task; a lane packs two
-// adjacent k into bf16 pairs (4-byte stores).
+// Lp padded lines.  k contiguous: a warp takes a (line, segment of PACK_SEG)
+// task.
 constexpr int PACK_SEG = 2048;
-__device__ __forceinline__ void ld_pair(const View& A, int64_t ro, bool live, int K,
-                                        int k0, int k, cplx& a0, cplx& a1) {
-  a0 = a1 = cmake(0, 0);
-  if (!live) return;
-  if (k < K) a0 = A.p[ro + vcol32(A, k0 + k)];
-  if (k + 1 < K) a1 = A.p[ro + vcol32(A, k0 + k + 1)];
-  if (A.conj) {
-    a0.y = -a0.y;
-    a1.y = -a1.y;
-  }
-}
-
-template <int S>
-__global__ void slice_pack_a(View A, int M, int K, int k0, int Mp, int Kp,
-                             int npairs, const int* __restrict__ eA,
-                             __nv_bfloat16* out) {
-  const int64_t ld = (int64_t)2 * npairs * Kp;
+template <int S, bool ISB>
+__global__ void __launch_bounds__(256)
+    slice_pack_kernel(View X, int L, int K, int k0, int Lp, int Kp,
+                      const int* __restrict__ eX, __nv_bfloat16* out) {
+  const int64_t ld = (int64_t)2 * S * Kp;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int nsg = (Kp + PACK_SEG - 1) / PACK_SEG;
-  const int64_t ntask = (int64_t)Mp * nsg;
-  for (int64_t t = warp; t < ntask; t += nwarp) {
-    const int m = (int)(t / nsg), k1 = (int)(t % nsg) * PACK_SEG;
+  for (int64_t t = warp; t < (int64_t)Lp * nsg; t += nwarp) {
+    const int l = (int)(t / nsg), k1 = (int)(t % nsg) * PACK_SEG;
     const int k2 = min(Kp, k1 + PACK_SEG);
-    const bool live = m < M;
-    const int64_t ro = live ? vrow(A, m) : 0;
-    const int e = live ? eA[m] : 0;
-    __nv_bfloat16* o = out + (int64_t)m * ld;
+    const bool live = l < L;
+    const cplx* x = X.p + (live ? vrow(X, l) : 0);
+    const int e = live ? eX[l] : 0;
+    __nv_bfloat16* o = out + (int64_t)l * (ISB ? 2 : 1) * ld;
     for (int k = k1 + 2 * lane; k < k2; k += 64) {
-      cplx a0, a1;
-      ld_pair(A, ro, live, K, k0, k, a0, a1);
-      __nv_bfloat16 r0[S], i0[S], r1[S], i1[S];
-      slices<S>(a0.x, e, r0);
-      slices<S>(a0.y, e, i0);
-      slices<S>(a1.x, e, r1);
-      slices<S>(a1.y, e, i1);
-      for (int p = 0; p < npairs; ++p) {
-        const int q = c_si[p];
-        *(__nv_bfloat162*)(o + (2 * p) * (int64_t)Kp + k) = __halves2bfloat162(r0[q], r1[q]);
-        *(__nv_bfloat162*)(o + (2 * p + 1) * (int64_t)Kp + k) =
-            __halves2bfloat162(i0[q], i1[q]);
+      cplx a0 = cmake(0, 0), a1 = cmake(0, 0);
+      if (live && k < K) a0 = x[vcol32(X, k0 + k)];
+      if (live && k + 1 < K) a1 = x[vcol32(X, k0 + k + 1)];
+      if (X.conj) {
+        a0.y = -a0.y;
+        a1.y = -a1.y;
       }
+      pack_two<S, ISB>(a0, a1, e, o + k, ld, Kp);
     }
   }
 }
 
-template <int S>
-__global__ void slice_pack_b(View B, int K, int k0, int N, int Np2, int Kp,
-                             int npairs, const int* __restrict__ eB,
-                             __nv_bfloat16* out) {
-  const int64_t ld = (int64_t)2 * npairs * Kp;
-  const int64_t total = (int64_t)(Np2 / 2) * Kp;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-       idx < total; idx += (int64_t)gridDim.x * blockDim.x) {
-    const int n = idx / Kp, k = idx % Kp;
-    cplx b = cmake(0, 0);
-    int e = 0;
-    if (n < N) {
-      e = eB[n];
-      if (k < K) {
-        b = B.p[vrow(B, k0 + k) + vcol(B, n)];
-        if (B.conj) b.y = -b.y;
-      }
+// Lines contiguous: a block takes tiles of 32 lines x 64 k, reads them along
+// the lines (512 bytes a warp) and packs them along k from shared memory.
+template <int S, bool ISB>
+__global__ void __launch_bounds__(256)
+    slice_pack_lines_kernel(View X, int L, int K, int k0, int Lp, int Kp,
+                            const int* __restrict__ eX, __nv_bfloat16* out) {
+  __shared__ cplx tile[64][33];
+  const int64_t ld = (int64_t)2 * S * Kp;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nkt = Kp / 64;
+  const int64_t ntask = (int64_t)((Lp + 31) / 32) * nkt;
+  for (int64_t t = blockIdx.x; t < ntask; t += gridDim.x) {
+    const int l0 = (int)(t / nkt) * 32, kt = (int)(t % nkt) * 64;
+    const bool live = l0 + lane < L;
+    const cplx* x = X.p + (live ? vrow(X, l0 + lane) : 0);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const int k = kt + warp + 8 * r;
+      cplx a = cmake(0, 0);
+      if (live && k < K) a = x[vcol32(X, k0 + k)];
+      if (X.conj) a.y = -a.y;
+      tile[warp + 8 * r][lane] = a;
     }
-    __nv_bfloat16 re[S], im[S];
-    slices<S>(b.x, e, re);
-    slices<S>(b.y, e, im);
-    __nv_bfloat16* o0 = out + (int64_t)(2 * n) * ld + k;
-    __nv_bfloat16* o1 = o0 + ld;
-    for (int p = 0; p < npairs; ++p) {
-      const int j = c_sj[p];
-      o0[(2 * p) * (int64_t)Kp] = re[j];
-      o0[(2 * p + 1) * (int64_t)Kp] = __hneg(im[j]);
-      o1[(2 * p) * (int64_t)Kp] = im[j];
-      o1[(2 * p + 1) * (int64_t)Kp] = re[j];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int l = l0 + warp * 4 + r;
+      if (l >= Lp) break;
+      const int e = l < L ? eX[l] : 0;
+      pack_two<S, ISB>(tile[2 * lane][l - l0], tile[2 * lane + 1][l - l0], e,
+                       out + (int64_t)l * (ISB ? 2 : 1) * ld + kt + 2 * lane, ld, Kp);
     }
   }
+}
+
+// exponents and packed slices of L lines (padded to Lp) of X over [k0, k0 + K)
+template <int S, bool ISB>
+void pack_lines(cudaStream_t s, View X, int L, int K, int k0, int Lp, int Kp, int* e,
+                size_t e_count, __nv_bfloat16* out) {
+  CVS_CUDA(cudaMemsetAsync(e, 0x80, e_count * sizeof(int), s));
+  // lanes go along the contiguous mode (along k when neither or both are)
+  const bool lines = X.cs_lo != 1 && X.rs_lo == 1 && (X.r_lo == INT32_MAX || X.r_lo >= 16);
+  if (lines) {
+    line_exp_kernel<false><<<warp_tasks_grid((L + 31) / 32, K, EXP_SEG_LINES), 256, 0, s>>>(
+        X, L, K, k0, e);
+    CVS_CHECK_LAUNCH();
+    const int64_t tiles = (int64_t)((Lp + 31) / 32) * (Kp / 64);
+    slice_pack_lines_kernel<S, ISB>
+        <<<(unsigned)std::min<int64_t>(tiles, 152 * 16), 256, 0, s>>>(X, L, K, k0, Lp, Kp, e,
+                                                                      out);
+  } else {
+    line_exp_kernel<true><<<warp_tasks_grid(L, K, EXP_SEG), 256, 0, s>>>(X, L, K, k0, e);
+    CVS_CHECK_LAUNCH();
+    slice_pack_kernel<S, ISB><<<warp_tasks_grid(Lp, Kp, PACK_SEG), 256, 0, s>>>(X, L, K, k0, Lp,
+                                                                               Kp, e, out);
+  }
+  CVS_CHECK_LAUNCH();
 }
 
 // ---------------------------------------------------------------------------
@@ -974,6 +1316,9 @@ __global__ void slice_pack_b(View B, int K, int k0, int N, int Np2, int Kp,
 // per K step instead of ten, and each A tile is read from shared memory
 // once.  The drain adds each order, times its scale, to float-float
 // accumulators.
+//
+// It serves the narrow and small products that the pairs of CTAs above would
+// pad (plan_slices).
 //
 // CTA: 576 threads, tile 128 x 64 (N' = 64: 32 complex columns).  Warp 0
 // lane 0: TMA producer; warp 1 lane 0: MMA issuer; warps 2..17: drain (warp
@@ -1167,90 +1512,26 @@ __global__ void __launch_bounds__(576, 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
 }
 
-// A'' [Mp][8 Kp]: segment 2 i + {0: re, 1: im} holds slice i; tasks as in
-// slice_pack_a
-__global__ void slice4r_pack_a(View A, int M, int K, int k0, int Mp, int Kp,
-                               const int* __restrict__ eA, __nv_bfloat16* out) {
-  const int64_t ld = (int64_t)8 * Kp;
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int nsg = (Kp + PACK_SEG - 1) / PACK_SEG;
-  const int64_t ntask = (int64_t)Mp * nsg;
-  for (int64_t t = warp; t < ntask; t += nwarp) {
-    const int m = (int)(t / nsg), k1 = (int)(t % nsg) * PACK_SEG;
-    const int k2 = min(Kp, k1 + PACK_SEG);
-    const bool live = m < M;
-    const int64_t ro = live ? vrow(A, m) : 0;
-    const int e = live ? eA[m] : 0;
-    __nv_bfloat16* o = out + (int64_t)m * ld;
-    for (int k = k1 + 2 * lane; k < k2; k += 64) {
-      cplx a0, a1;
-      ld_pair(A, ro, live, K, k0, k, a0, a1);
-      __nv_bfloat16 r0[4], i0[4], r1[4], i1[4];
-      slices<4>(a0.x, e, r0);
-      slices<4>(a0.y, e, i0);
-      slices<4>(a1.x, e, r1);
-      slices<4>(a1.y, e, i1);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        *(__nv_bfloat162*)(o + (2 * i) * (int64_t)Kp + k) = __halves2bfloat162(r0[i], r1[i]);
-        *(__nv_bfloat162*)(o + (2 * i + 1) * (int64_t)Kp + k) = __halves2bfloat162(i0[i], i1[i]);
-      }
-    }
-  }
-}
-
-// B'' [Np2][8 Kp]: rows 2n and 2n + 1, segment 2 j + {0, 1} of slice j
-__global__ void slice4r_pack_b(View B, int K, int k0, int N, int Np2, int Kp,
-                               const int* __restrict__ eB, __nv_bfloat16* out) {
-  const int64_t ld = (int64_t)8 * Kp;
-  const int64_t total = (int64_t)(Np2 / 2) * Kp;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int n = (int)(idx / Kp), k = (int)(idx % Kp);
-    cplx b = cmake(0, 0);
-    int e = 0;
-    if (n < N) {
-      e = eB[n];
-      if (k < K) {
-        b = B.p[vrow(B, k0 + k) + vcol(B, n)];
-        if (B.conj) b.y = -b.y;
-      }
-    }
-    __nv_bfloat16 re[4], im[4];
-    slices<4>(b.x, e, re);
-    slices<4>(b.y, e, im);
-    __nv_bfloat16* o0 = out + (int64_t)(2 * n) * ld + k;
-    __nv_bfloat16* o1 = o0 + ld;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      o0[(2 * j) * (int64_t)Kp] = re[j];
-      o0[(2 * j + 1) * (int64_t)Kp] = __hneg(im[j]);
-      o1[(2 * j) * (int64_t)Kp] = im[j];
-      o1[(2 * j + 1) * (int64_t)Kp] = re[j];
-    }
-  }
-}
-
-// packed geometry: SLICE4 packs each slice once (8 segments, N' tiles of
-// 64, the slice-reuse kernel); SLICE7 packs one segment pair per slice pair
-// (56 segments, N' tiles of 128).  K runs in chunks of kc so that the packs
-// of a chunk stay within PACK_BUDGET; a B operand held in a cache is packed
-// once over its whole K (KpF) and only A's pack counts against the budget.
+// packed geometry: every slice once (2 segments each), rows padded to the
+// tiles.  K runs in chunks of kc, each with its own exponents; a B operand
+// held in a cache is packed once over its whole K (KpF) and only A's pack
+// counts against the budget.  kc is what PACK_BUDGET holds at 8 (SLICE4) or
+// 56 (SLICE7) segments: a chunk's length is also the reach of its exponents,
+// so the 7-slice chunks stay as short as when every slice pair had segments
+// of its own.
 struct SDims {
-  int Mp, Np2, npairs, nseg, kc, KpF;
+  int Mp, Np2, nseg, cseg, kc, KpF;
   size_t a_bytes, b_bytes, e_bytes;
 };
 SDims sdims_of(int M, int N, int K, int nslices, bool b_cached, bool a_cached = false) {
   SDims d;
-  const int tn = nslices == 4 ? RBN : SBN;
+  const int tn = nslices == 4 ? RBN : 128;
   d.Mp = (M + BM - 1) / BM * BM;
   d.Np2 = (2 * N + tn - 1) / tn * tn;
-  d.npairs = nslices * (nslices + 1) / 2;
-  d.nseg = nslices == 4 ? 8 : 2 * d.npairs;
+  d.nseg = 2 * nslices;
+  d.cseg = nslices == 4 ? 8 : nslices * (nslices + 1);
   d.KpF = (int)(((int64_t)K + BK - 1) / BK * BK);
-  const size_t per_k = (size_t)((a_cached ? 0 : d.Mp) + (b_cached ? 0 : d.Np2)) * d.nseg * 2;
+  const size_t per_k = (size_t)((a_cached ? 0 : d.Mp) + (b_cached ? 0 : d.Np2)) * d.cseg * 2;
   int64_t kc = per_k ? (int64_t)(PACK_BUDGET / per_k) / BK * BK : (int64_t)d.KpF;
   kc = std::max<int64_t>(kc, BK);
   d.kc = (int)std::min<int64_t>(kc, d.KpF);
@@ -1258,6 +1539,56 @@ SDims sdims_of(int M, int N, int K, int nslices, bool b_cached, bool a_cached = 
   d.b_bytes = b_cached ? 0 : (size_t)d.Np2 * d.nseg * d.kc * 2;
   d.e_bytes = ((size_t)d.Mp + d.Np2 / 2 + 64) * sizeof(int);
   return d;
+}
+
+// How a product of nkb K blocks is laid out on the GPU, by modelled time in
+// us.  Pairs of CTAs: 1.8 (4 slices) or 2.75 (7) us per unit of a tile, tiles
+// (times K slices) dealt out to 76 pairs, about 7 units of start and end.
+// SLICE4's 128 x 64 tiles: 1.3 us per unit, a CTA per tile, 8 units of start
+// and end: they keep narrow (2 N <= 64) and small products.  K slices need
+// an output that fits the scratch, and cost its way through memory (32 bytes
+// per partial at 6 TB/s) and a launch.
+struct SlicePlan {
+  bool pair;
+  int splits;
+};
+SlicePlan plan_slices(int nslices, int M, int N, int nkb, size_t part_elems) {
+  SlicePlan best{true, 1};
+  double tbest = 1e300;
+  auto consider = [&](bool pair, double tiles, double workers, double unit, double fixed) {
+    for (int sp = 1; sp <= 32; ++sp) {
+      if (sp > 1 && (nkb / sp < 4 || (size_t)sp * M * N > part_elems)) break;
+      const double units = 2.0 * ((nkb + sp - 1) / sp);
+      double t = std::ceil(tiles * sp / workers) * (units + fixed) * unit;
+      if (sp > 1) t += 3.0 + 32.0 * sp * (double)M * N / 6e6;
+      if (t < tbest) {
+        tbest = t;
+        best = SlicePlan{pair, sp};
+      }
+    }
+  };
+  const int pn = nslices == 4 ? PairCfg<4>::PN : PairCfg<7>::PN;
+  const double tm = (M + P_BM - 1) / P_BM, tn = (2 * N + pn - 1) / pn;
+  consider(true, tm * tn, 76.0, nslices == 4 ? 1.8 : 2.75, 7.0);
+  if (nslices == 4)
+    consider(false, (double)((M + BM - 1) / BM) * ((2 * N + RBN - 1) / RBN), 152.0, 1.3, 8.0);
+  return best;
+}
+
+template <int NS>
+void launch_pair(cudaStream_t s, const CUtensorMap& ma, const CUtensorMap& mb,
+                 const CUtensorMap& mb2, int kpa,
+                 int ka_off, int kpb, int kb_off, int nkb, int zl, int nz, int M, int N,
+                 const int* eA, const int* eB, double alpha, double beta, View C, cplx* part,
+                 int* err) {
+  const int ntm = (M + P_BM - 1) / P_BM, ntn = (2 * N + PairCfg<NS>::PN - 1) / PairCfg<NS>::PN;
+  const int64_t items = (int64_t)ntm * ntn * nz;
+  CVS_REQUIRE(items <= INT32_MAX, -1, "zgemm_slice: output too large");
+  const unsigned grid = 2 * (unsigned)std::min<int64_t>(items, 76);
+  tc_slice_pair_kernel<NS><<<grid, pair_threads<NS>(), pair_smem<NS>(), s>>>(
+      ma, mb, mb2, kpa, ka_off, kpb, kb_off, nkb, zl, ntm, ntn, (int)items, M, N, eA, eB, alpha, beta,
+      C, part, err);
+  CVS_CHECK_LAUNCH();
 }
 
 }  // namespace
@@ -1287,8 +1618,8 @@ size_t slice_bcache_bytes(int N, int K, int nslices) {
 int64_t slice_row_slab(int M, int N, int K, int nslices) {
   SDims d = sdims_of(M, N, K, nslices, false);
   if (d.kc >= d.KpF) return M;  // K is whole already
-  const size_t per_row = (size_t)d.nseg * d.KpF * 2;
-  const size_t bfull = (size_t)d.Np2 * d.nseg * d.KpF * 2;
+  const size_t per_row = (size_t)d.cseg * d.KpF * 2;
+  const size_t bfull = (size_t)d.Np2 * d.cseg * d.KpF * 2;
   if (bfull >= PACK_BUDGET / 2) return M;
   const int64_t rows = (int64_t)((PACK_BUDGET - bfull) / per_row) / BM * BM;
   return rows >= 16 * BM ? rows : M;
@@ -1306,34 +1637,36 @@ void zgemm_slice(cudaStream_t s, int nslices, int M, int N, int K,
               "zgemm_slice: workspace too small");
   static std::once_flag attr;
   std::call_once(attr, [] {
-    cudaFuncSetAttribute(tc_slice_kernel,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, S_SMEM);
+    cudaFuncSetAttribute(tc_slice_pair_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         pair_smem<4>());
+    cudaFuncSetAttribute(tc_slice_pair_kernel<7>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         pair_smem<7>());
     cudaFuncSetAttribute(tc_slice4r_kernel,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, R_SMEM);
   });
+  auto pack_a = [&](int Kc, int k0, int Kp, int* e, __nv_bfloat16* out) {
+    if (nslices == 4)
+      pack_lines<4, false>(s, A, M, Kc, k0, d.Mp, Kp, e, d.Mp, out);
+    else
+      pack_lines<7, false>(s, A, M, Kc, k0, d.Mp, Kp, e, d.Mp, out);
+  };
+  const size_t eb_n = (size_t)d.Np2 / 2 + 64;
+  auto pack_b = [&](int Kc, int k0, int Kp, int* e, __nv_bfloat16* out) {
+    if (nslices == 4)
+      pack_lines<4, true>(s, trans(B), N, Kc, k0, d.Np2 / 2, Kp, e, eb_n, out);
+    else
+      pack_lines<7, true>(s, trans(B), N, Kc, k0, d.Np2 / 2, Kp, e, eb_n, out);
+  };
   __nv_bfloat16* ap = (__nv_bfloat16*)work;
   __nv_bfloat16* bp = (__nv_bfloat16*)((char*)work + d.a_bytes);
   int* eA = (int*)((char*)work + d.a_bytes + d.b_bytes);
   int* eB = eA + d.Mp;
-  const bool reuse = nslices == 4;
-  const int64_t tiles = (int64_t)(d.Np2 / (reuse ? RBN : SBN)) * (d.Mp / BM);
-  const size_t eb_n = (size_t)d.Np2 / 2 + 64;
   const size_t bfull = (size_t)d.Np2 * d.nseg * d.KpF * 2;
   if (bc) {
     // the cached B: packed once over the whole K, with whole-column exponents
     CVS_REQUIRE(bc->bytes >= bfull + eb_n * sizeof(int), -1, "zgemm_slice: B cache too small");
     if (!bc->filled) {
-      int* ec = (int*)((char*)bc->base + bfull);
-      __nv_bfloat16* bq = (__nv_bfloat16*)bc->base;
-      CVS_CUDA(cudaMemsetAsync(ec, 0x80, eb_n * sizeof(int), s));
-      col_exp_kernel<<<warp_tasks_grid(N, K, EXP_SEG), 256, 0, s>>>(B, K, 0, N, ec);
-      CVS_CHECK_LAUNCH();
-      const unsigned gb = grid1d((int64_t)(d.Np2 / 2) * d.KpF, 256);
-      if (reuse)
-        slice4r_pack_b<<<gb, 256, 0, s>>>(B, K, 0, N, d.Np2, d.KpF, ec, bq);
-      else
-        slice_pack_b<7><<<gb, 256, 0, s>>>(B, K, 0, N, d.Np2, d.KpF, d.npairs, ec, bq);
-      CVS_CHECK_LAUNCH();
+      pack_b(K, 0, d.KpF, (int*)((char*)bc->base + bfull), (__nv_bfloat16*)bc->base);
       bc->filled = true;
     }
   }
@@ -1343,13 +1676,7 @@ void zgemm_slice(cudaStream_t s, int nslices, int M, int N, int K,
     CVS_REQUIRE(ac->bytes >= afull + (size_t)d.Mp * sizeof(int), -1,
                 "zgemm_slice: A cache too small");
     if (!ac->filled) {
-      int* ea = (int*)((char*)ac->base + afull);
-      CVS_CUDA(cudaMemsetAsync(ea, 0x80, (size_t)d.Mp * sizeof(int), s));
-      row_exp_kernel<<<warp_tasks_grid(M, K, EXP_SEG), 256, 0, s>>>(A, M, K, 0, ea);
-      CVS_CHECK_LAUNCH();
-      slice4r_pack_a<<<warp_tasks_grid(d.Mp, d.KpF, PACK_SEG), 256, 0, s>>>(
-          A, M, K, 0, d.Mp, d.KpF, ea, (__nv_bfloat16*)ac->base);
-      CVS_CHECK_LAUNCH();
+      pack_a(K, 0, d.KpF, (int*)((char*)ac->base + afull), (__nv_bfloat16*)ac->base);
       ac->filled = true;
     }
   }
@@ -1366,68 +1693,32 @@ void zgemm_slice(cudaStream_t s, int nslices, int M, int N, int K,
     const __nv_bfloat16* apc = ac ? (const __nv_bfloat16*)ac->base : ap;
     const int* eAc = ac ? (const int*)((const char*)ac->base + afull) : eA;
     const int kpa = ac ? d.KpF : Kp, ka_off = ac ? k0 / BK : 0;
-    if (!ac) {
-      CVS_CUDA(cudaMemsetAsync(eA, 0x80, (size_t)d.Mp * sizeof(int), s));
-      row_exp_kernel<<<warp_tasks_grid(M, Kc, EXP_SEG), 256, 0, s>>>(A, M, Kc, k0, eA);
-      CVS_CHECK_LAUNCH();
-    }
-    if (!bc) {
-      CVS_CUDA(cudaMemsetAsync(eB, 0x80, eb_n * sizeof(int), s));
-      col_exp_kernel<<<warp_tasks_grid(N, Kc, EXP_SEG), 256, 0, s>>>(B, Kc, k0, N, eB);
-      CVS_CHECK_LAUNCH();
-    }
-    const unsigned ga = warp_tasks_grid(d.Mp, Kp, PACK_SEG);
-    const unsigned gb = grid1d((int64_t)(d.Np2 / 2) * Kp, 256);
-    if (reuse) {
-      if (!ac) {
-        slice4r_pack_a<<<ga, 256, 0, s>>>(A, M, Kc, k0, d.Mp, Kp, eA, ap);
-        CVS_CHECK_LAUNCH();
-      }
-      if (!bc) {
-        slice4r_pack_b<<<gb, 256, 0, s>>>(B, Kc, k0, N, d.Np2, Kp, eB, bp);
-        CVS_CHECK_LAUNCH();
-      }
-    } else {
-      slice_pack_a<7><<<ga, 256, 0, s>>>(A, M, Kc, k0, d.Mp, Kp, d.npairs, eA, ap);
-      CVS_CHECK_LAUNCH();
-      if (!bc) {
-        slice_pack_b<7><<<gb, 256, 0, s>>>(B, Kc, k0, N, d.Np2, Kp, d.npairs, eB, bp);
-        CVS_CHECK_LAUNCH();
-      }
-    }
-    const int64_t kcols = (int64_t)d.nseg * Kp, kcols_b = (int64_t)d.nseg * kpb;
+    if (!ac) pack_a(Kc, k0, Kp, eA, ap);
+    if (!bc) pack_b(Kc, k0, Kp, eB, bp);
     const double beta_c = (k0 == 0) ? beta : 1.0;
-    if (reuse) {
-      CUtensorMap ma = make_map(apc, d.Mp, (int64_t)d.nseg * kpa, BM);
-      CUtensorMap mb = make_map(bpc, d.Np2, kcols_b, RBN);
-      const int nkb = Kp / BK;  // K blocks; a run spans two
-      int sp = tc_splits(tiles, nkb, 2 * (R_RUN / 2));
-      if (part == nullptr || (size_t)sp * M * N > part_elems) sp = 1;
-      const int zl = (nkb + sp - 1) / sp;
-      const int nz = (nkb + zl - 1) / zl;
-      dim3 grid(d.Np2 / RBN, d.Mp / BM, nz);
-      const int tok = kstats_begin(s, K_TC_SLICE, 8.0 * M * N * (double)Kc);
-      tc_slice4r_kernel<<<grid, 576, R_SMEM, s>>>(ma, mb, kpa, ka_off, kpb, kb_off, nkb, zl,
-                                                  M, N, eAc, eBc, alpha, beta_c, C,
-                                                  nz > 1 ? part : nullptr, err);
-      CVS_CHECK_LAUNCH();
-      kstats_end(s, tok);
-      if (nz > 1) splitk_reduce(s, M, N, nz, part, beta_c, C);
-      continue;
-    }
-    CUtensorMap ma = make_map(ap, d.Mp, kcols, BM);
-    CUtensorMap mb = make_map(bpc, d.Np2, kcols_b, SBN);
-    const int ktpp = 2 * Kp / BK;
-    int sp = tc_splits(tiles, ktpp, RUN_KT);
-    if (part == nullptr || (size_t)sp * M * N > part_elems) sp = 1;
-    const int zl = (ktpp + sp - 1) / sp;
-    const int nz = (ktpp + zl - 1) / zl;
-    dim3 grid(d.Np2 / SBN, d.Mp / BM, nz);
+    const int nkb = Kp / BK;  // K blocks
+    const SlicePlan pl = plan_slices(nslices, M, N, nkb, part ? part_elems : 0);
+    const int zl = (nkb + pl.splits - 1) / pl.splits;
+    const int nz = (nkb + zl - 1) / zl;
+    cplx* pp = nz > 1 ? part : nullptr;
+    CUtensorMap ma = make_map(apc, d.Mp, (int64_t)d.nseg * kpa, BM);
+    // boxes of 64 rows: half a 128-column slice (4 slices) or a whole
+    // 64-column one; of 32 rows: half of that
+    CUtensorMap mb = make_map(bpc, d.Np2, (int64_t)d.nseg * kpb, 64);
+    CUtensorMap mb2 = make_map(bpc, d.Np2, (int64_t)d.nseg * kpb, 32);
     const int tok = kstats_begin(s, K_TC_SLICE, 8.0 * M * N * (double)Kc);
-    tc_slice_kernel<<<grid, 576, S_SMEM, s>>>(ma, mb, d.npairs, ktpp, kpb, kb_off, zl, M, N,
-                                              eA, eBc, alpha, beta_c, C,
-                                              nz > 1 ? part : nullptr, err);
-    CVS_CHECK_LAUNCH();
+    if (pl.pair && nslices == 4) {
+      launch_pair<4>(s, ma, mb, mb2, kpa, ka_off, kpb, kb_off, nkb, zl, nz, M, N, eAc, eBc, alpha,
+                     beta_c, C, pp, err);
+    } else if (pl.pair) {
+      launch_pair<7>(s, ma, mb, mb2, kpa, ka_off, kpb, kb_off, nkb, zl, nz, M, N, eAc, eBc, alpha,
+                     beta_c, C, pp, err);
+    } else {
+      dim3 grid(d.Np2 / RBN, d.Mp / BM, nz);
+      tc_slice4r_kernel<<<grid, 576, R_SMEM, s>>>(ma, mb, kpa, ka_off, kpb, kb_off, nkb, zl, M, N,
+                                                  eAc, eBc, alpha, beta_c, C, pp, err);
+      CVS_CHECK_LAUNCH();
+    }
     kstats_end(s, tok);
     if (nz > 1) splitk_reduce(s, M, N, nz, part, beta_c, C);
   }

@@ -59,7 +59,7 @@ template <int TY, int TX, int RM, int RN, int BK, int ST>
 __global__ void __launch_bounds__(NT)
     zgemm_f64_kernel(int M, int N, int K, double alpha, View A, View B,
                      double beta, View C, int a_kfast, int b_kfast,
-                     int ntn, int kchunk, cplx* part) {
+                     int ntn, int kchunk, int period, cplx* part) {
   constexpr int KX = NT / (TY * TX);
   constexpr int TM = TY * RM, TN = TX * RN;
   constexpr int EA = (TM * BK + NT - 1) / NT, EB = (TN * BK + NT - 1) / NT;
@@ -132,13 +132,26 @@ __global__ void __launch_bounds__(NT)
     }
   };
 
-  double accr[RM][RN], acci[RM][RN];
+  // every `period` steps the sums so far are added up apart: the rounding
+  // error of a chain of additions grows with its length
+  double accr[RM][RN], acci[RM][RN], sumr[RM][RN], sumi[RM][RN];
 #pragma unroll
   for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < RN; ++j) accr[i][j] = acci[i][j] = 0.0;
+    for (int j = 0; j < RN; ++j) accr[i][j] = acci[i][j] = sumr[i][j] = sumi[i][j] = 0.0;
+  auto flush = [&]() {
+#pragma unroll
+    for (int i = 0; i < RM; ++i)
+#pragma unroll
+      for (int j = 0; j < RN; ++j) {
+        sumr[i][j] += accr[i][j];
+        sumi[i][j] += acci[i][j];
+        accr[i][j] = acci[i][j] = 0.0;
+      }
+  };
 
   const int ntiles = (ke - kb + BK - 1) / BK;
+  int left = period;
   // one copy group per step, empty past the end, so that a fixed count of
   // pending groups says that step t has landed
 #pragma unroll
@@ -172,7 +185,12 @@ __global__ void __launch_bounds__(NT)
           acci[i][j] = fma(a[i].y, b[j].x, acci[i][j]);
         }
     }
+    if (--left == 0) {
+      flush();
+      left = period;
+    }
   }
+  flush();
 
   auto put = [&](int r, int c, double re, double im) {
     if (r >= M || c >= N) return;
@@ -195,7 +213,7 @@ __global__ void __launch_bounds__(NT)
     for (int i = 0; i < RM; ++i)
 #pragma unroll
       for (int j = 0; j < RN; ++j)
-        sh[(kx * TM + ty + TY * i) * TN + tx + TX * j] = cmake(accr[i][j], acci[i][j]);
+        sh[(kx * TM + ty + TY * i) * TN + tx + TX * j] = cmake(sumr[i][j], sumi[i][j]);
     __syncthreads();
     for (int e = tid; e < TM * TN; e += NT) {
       double re = 0.0, im = 0.0;
@@ -211,36 +229,39 @@ __global__ void __launch_bounds__(NT)
     for (int i = 0; i < RM; ++i)
 #pragma unroll
       for (int j = 0; j < RN; ++j)
-        put(m0 + ty + TY * i, n0 + tx + TX * j, accr[i][j], acci[i][j]);
+        put(m0 + ty + TY * i, n0 + tx + TX * j, sumr[i][j], sumi[i][j]);
   }
 }
 
 typedef void (*F64Kernel)(int, int, int, double, View, View, double, View, int, int, int, int,
-                          cplx*);
+                          int, cplx*);
 struct F64Shape {
-  int tm, tn, bk, kx;
+  int tm, tn, bk;
+  double eff;
   F64Kernel fn;
 };
-#define CVS_F64(TY, TX, RM, RN, BK, ST) \
-  {TY * RM, TX * RN, BK, NT / (TY * TX), zgemm_f64_kernel<TY, TX, RM, RN, BK, ST>}
+#define CVS_F64(TY, TX, RM, RN, BK, ST, EFF) \
+  {TY * RM, TX * RN, BK, EFF, zgemm_f64_kernel<TY, TX, RM, RN, BK, ST>}
+// with the share of the FP64 rate each holds on 1000 products of 246 x 165 x
+// 200 (its padding and whole k steps counted as work)
 const F64Shape F64_SHAPES[] = {
-    CVS_F64(16, 8, 2, 4, 16, 2),  // 32 x 32
-    CVS_F64(16, 8, 2, 3, 16, 2),  // 32 x 24
-    CVS_F64(16, 8, 2, 2, 16, 3),  // 32 x 16
-    CVS_F64(32, 4, 1, 3, 16, 3),  // 32 x 12
-    CVS_F64(32, 4, 1, 2, 16, 4),  // 32 x 8
-    CVS_F64(16, 8, 1, 2, 16, 4),  // 16 x 16
-    CVS_F64(16, 8, 1, 1, 16, 4),  // 16 x 8
-    CVS_F64(32, 2, 1, 3, 16, 4),  // 32 x 6
-    CVS_F64(32, 4, 1, 1, 16, 4),  // 32 x 4
-    CVS_F64(32, 2, 1, 1, 16, 4),  // 32 x 2
-    CVS_F64(32, 1, 1, 1, 16, 4),  // 32 x 1
-    CVS_F64(8, 8, 1, 1, 16, 4),   // 8 x 8
-    CVS_F64(8, 4, 1, 1, 32, 3),   // 8 x 4
-    CVS_F64(4, 32, 1, 1, 16, 4),  // 4 x 32
-    CVS_F64(2, 32, 3, 1, 16, 4),  // 6 x 32
-    CVS_F64(4, 4, 3, 3, 16, 4),   // 12 x 12
-    CVS_F64(2, 2, 3, 3, 32, 3),   // 6 x 6
+    CVS_F64(16, 8, 2, 4, 16, 2, 0.96),  // 32 x 32
+    CVS_F64(16, 8, 2, 3, 16, 2, 0.95),  // 32 x 24
+    CVS_F64(16, 8, 2, 2, 16, 3, 0.95),  // 32 x 16
+    CVS_F64(32, 4, 1, 3, 16, 3, 0.95),  // 32 x 12
+    CVS_F64(32, 4, 1, 2, 16, 4, 0.91),  // 32 x 8
+    CVS_F64(16, 8, 1, 2, 16, 4, 0.91),  // 16 x 16
+    CVS_F64(16, 8, 1, 1, 16, 4, 0.91),  // 16 x 8
+    CVS_F64(32, 2, 1, 3, 16, 4, 0.98),  // 32 x 6
+    CVS_F64(32, 4, 1, 1, 16, 4, 0.95),  // 32 x 4
+    CVS_F64(32, 2, 1, 1, 16, 4, 0.90),  // 32 x 2
+    CVS_F64(32, 1, 1, 1, 16, 4, 0.82),  // 32 x 1
+    CVS_F64(8, 8, 1, 1, 16, 4, 0.91),   // 8 x 8
+    CVS_F64(8, 4, 1, 1, 32, 3, 0.83),   // 8 x 4
+    CVS_F64(4, 32, 1, 1, 16, 4, 0.95),  // 4 x 32
+    CVS_F64(2, 32, 3, 1, 16, 4, 0.98),  // 6 x 32
+    CVS_F64(4, 4, 3, 3, 16, 4, 0.95),   // 12 x 12
+    CVS_F64(2, 2, 3, 3, 32, 3, 0.74),   // 6 x 6
 };
 #undef CVS_F64
 
@@ -250,10 +271,10 @@ struct F64Plan {
 };
 
 // The tile shape and number of K slices with the least modelled time, in SM
-// cycles.  A block's FMAs take w = 2 tm tn ceil(K / s) cycles of its SM's
-// FP64 pipe (padding included), its set-up, stores and k-group sums about
-// 200 + 300 kx more; the SM with the most blocks sets the time, and one
-// block alone takes w plus 1000 cycles of latency per k step.  K slices
+// cycles.  A block's FMAs take w = 2 tm tn (k of whole steps) / eff cycles of
+// its SM's FP64 pipe (padding included), its set-up and stores about 200
+// more; the SM with the most blocks sets the time, and one block alone takes
+// w plus 1000 cycles of latency per k step.  K slices
 // cost one more launch (5000 cycles) and their partials' way through memory,
 // 32 bytes each at 3 KB per cycle.  The modelled time is within 5 % of the
 // measured one over these shapes at 61 x 47 x 83 to 1024^3 and 6 x 6 x 10^6.
@@ -272,9 +293,9 @@ F64Plan plan_f64(int M, int N, int K, int batch, size_t part_elems) {
     const double tiles = (double)((M + f.tm - 1) / f.tm) * ((N + f.tn - 1) / f.tn) * batch;
     for (int64_t s = 1; s == 1 || s <= smax; s *= 2) {
       const double ks = (double)((K + s - 1) / s);
-      const double w = 2.0 * f.tm * f.tn * ks;
-      double t = std::max(std::ceil(tiles * s / SMS) * (w + 200.0 + 300.0 * (f.kx - 1)),
-                          w + 1000.0 * std::ceil(ks / f.bk));
+      const double steps = std::ceil(ks / f.bk);
+      const double w = 2.0 * f.tm * f.tn * f.bk * steps / f.eff;
+      double t = std::max(std::ceil(tiles * s / SMS) * (w + 200.0), w + 1000.0 * steps);
       if (s > 1) t += 5000.0 + 32.0 * s * (double)M * N / 3000.0;
       if (t < tbest) {
         tbest = t;
@@ -347,12 +368,16 @@ void zgemm_f64(cudaStream_t s, int M, int N, int K, double alpha, View A,
   const int bk = p.shape->bk;
   const int kchunk = ((K + p.splits - 1) / p.splits + bk - 1) / bk * bk;
   const int nz = (K + kchunk - 1) / kchunk;
+  // long contractions in chains of 128 (45 x 60 x 5000: 6.1e-16 of the result
+  // in chains of 625, 3.1e-16 in these); short ones as they come (two more
+  // additions per output cost up to 8 % of the small tiles at K = 200)
+  const int period = K >= 4096 ? 128 / bk : INT32_MAX;
   const int ntn = (N + p.shape->tn - 1) / p.shape->tn;
   const int64_t tiles = (int64_t)ntn * ((M + p.shape->tm - 1) / p.shape->tm);
   CVS_REQUIRE(tiles <= INT32_MAX, -1, "zgemm_f64: output too large");
   dim3 grid((unsigned)tiles, 1, nz > 1 ? nz : batch);
   p.shape->fn<<<grid, NT, 0, s>>>(M, N, K, alpha, A, B, beta, C, a_kfast, b_kfast, ntn, kchunk,
-                                  nz > 1 ? part : nullptr);
+                                  period, nz > 1 ? part : nullptr);
   CVS_CHECK_LAUNCH();
   kstats_end(s, tok);
   if (nz > 1) splitk_reduce(s, M, N, nz, part, beta, C);

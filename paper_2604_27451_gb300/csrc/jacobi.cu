@@ -203,7 +203,9 @@ __device__ __forceinline__ void rotation(cplx apq, double app, double aqq, doubl
   c = 1.0;
   sv = cmake(0.0, 0.0);
   const double r = hypot(apq.x, apq.y);
-  if (!(r > 1e-300 && r > 1e-18 * sqrt(fabs(app * aqq)))) return;
+  // (the square root only where the squares do not tell)
+  const double r2 = r * r, pq = fabs(app * aqq);
+  if (!(r > 1e-300) || (!(r2 > 2e-36 * pq && r2 > 1e-290) && !(r > 1e-18 * sqrt(pq)))) return;
   const double tau = (aqq - app) / (2.0 * r);
   const double t = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
   c = 1.0 / sqrt(1.0 + t * t);
@@ -211,66 +213,33 @@ __device__ __forceinline__ void rotation(cplx apq, double app, double aqq, doubl
   sv = cmake(sn * apq.x / r, sn * apq.y / r);
 }
 
-// One step: An = J^H A J and V = V J for all pairs of the step.
-//
-// What bounds it: the FP64 pipes (two FMAs per SM and cycle), launch and
-// latency at small n.  A is only read, so a block takes a tile of JT x JT
-// pairs, computes their rotations and both sides of its (2 JT)^2 elements in
-// one pass (48 FP64 operations per 2 x 2 block, ~150 per rotation) and
-// writes them to An: one launch a step and one pass over A instead of three
-// and two.  Blocks from na on rotate JT pairs of columns of VR rows of V.
-// The rotations are worked out again in every block, so the larger tile
-// takes over where blocks outnumber the SMs.
-// A launch a step, measured against three: n = 600 24 us (33 us),
-// n = 240 11.6 us (20 us), n = 200 against one CTA 11 us (~190 us).
-template <int JT, int VR>
-__global__ void __launch_bounds__(JT * JT)
-    jstep_kernel(const cplx* __restrict__ A, cplx* __restrict__ An, cplx* __restrict__ V,
-                 int n, int np, int s, int nt, int na) {
-  __shared__ double cc[2 * JT];
-  __shared__ cplx se[2 * JT];
-  __shared__ int ip[2 * JT], iq[2 * JT];
-  const int tid = threadIdx.x, ti = tid / JT, tj = tid % JT;
-  const bool vblk = (int)blockIdx.x >= na;
-  const int blk = vblk ? (int)blockIdx.x - na : (int)blockIdx.x;
-  const int tk = blk / nt, tl = blk % nt;  // tk of a V block: its tile of rows
-  // pairs of the tile's columns at [0, JT), of its rows at [JT, 2 JT)
-  if (tid < 2 * JT) {
-    const int k = (tid < JT ? tl : tk) * JT + tid % JT;
-    int p = n, q = n;
-    if (k < np / 2 && !(vblk && tid >= JT)) rr_pair(k, np, s, p, q);
-    double c = 1.0;
-    cplx sv = cmake(0.0, 0.0);
-    if (q < n)
-      rotation(A[(int64_t)p * n + q], A[(int64_t)p * n + p].x, A[(int64_t)q * n + q].x, c, sv);
-    cc[tid] = c;
-    se[tid] = sv;
-    ip[tid] = p;
-    iq[tid] = q;
-  }
-  __syncthreads();
-  const int pl = ip[tj], ql = iq[tj];
-  const double cl = cc[tj];
-  const cplx sl = se[tj];
-  if (vblk) {
-    if (ql >= n || (sl.x == 0.0 && sl.y == 0.0)) return;
-    for (int r = tk * VR + ti; r < min(n, (tk + 1) * VR); r += JT) {
-      cplx* v = V + (int64_t)r * n;
-      const cplx vp = v[pl], vq = v[ql];
-      v[pl] = csub(cscale(vp, cl), cmul(cconj(sl), vq));
-      v[ql] = cadd(cmul(sl, vp), cscale(vq, cl));
-    }
-    return;
-  }
-  const int pk = ip[JT + ti], qk = iq[JT + ti];
-  const double ck = cc[JT + ti];
-  const cplx sk = se[JT + ti];
+struct Rot {
+  cplx s;
+  double c, pad;
+};
+// the rotation of pair k of step s, and its indices (p = n: no such pair)
+__device__ __forceinline__ Rot rotation_of(const cplx* A, int n, int np, int s, int k, int& p,
+                                           int& q) {
+  Rot r{cmake(0.0, 0.0), 1.0, 0.0};
+  p = q = n;
+  if (k < np / 2) rr_pair(k, np, s, p, q);
+  if (q < n)
+    rotation(A[(int64_t)p * n + q], A[(int64_t)p * n + p].x, A[(int64_t)q * n + q].x, r.c, r.s);
+  return r;
+}
+
+// An = J^H A J on the 2 x 2 block of rows (pk, qk) and columns (pl, ql)
+__device__ __forceinline__ void rotate_block(const cplx* __restrict__ A, cplx* __restrict__ An,
+                                             int n, int pk, int qk, const Rot& rk, int pl, int ql,
+                                             const Rot& rl) {
   auto get = [&](int r, int c) {
     return r < n && c < n ? A[(int64_t)r * n + c] : cmake(0.0, 0.0);
   };
   auto put = [&](int r, int c, cplx v) {
     if (r < n && c < n) An[(int64_t)r * n + c] = v;
   };
+  const double ck = rk.c, cl = rl.c;
+  const cplx sk = rk.s, sl = rl.s;
   cplx a = get(pk, pl), b = get(pk, ql), c = get(qk, pl), d = get(qk, ql);
   if (sk.x != 0.0 || sk.y != 0.0) {  // rows: p' = c p - s q, q' = conj(s) p + c q
     const cplx a0 = a, b0 = b;
@@ -290,6 +259,79 @@ __global__ void __launch_bounds__(JT * JT)
   put(pk, ql, b);
   put(qk, pl, c);
   put(qk, ql, d);
+}
+
+// columns (p, q) of the rows r0, r0 + dr, .. < r1 of V: V <- V J
+__device__ __forceinline__ void rotate_rows(cplx* V, int n, int p, int q, const Rot& r, int r0,
+                                            int r1, int dr) {
+  if (q >= n || (r.s.x == 0.0 && r.s.y == 0.0)) return;
+  for (int i = r0; i < r1; i += dr) {
+    cplx* v = V + (int64_t)i * n;
+    const cplx vp = v[p], vq = v[q];
+    v[p] = csub(cscale(vp, r.c), cmul(cconj(r.s), vq));
+    v[q] = cadd(cmul(r.s, vp), cscale(vq, r.c));
+  }
+}
+
+// One step as one launch: An = J^H A J and V = V J for all pairs of step s.
+// A is only read, so a block takes a tile of 8 x 8 pairs, computes their
+// rotations and both sides of its 16 x 16 elements in one pass; blocks from
+// na on rotate 8 pairs of columns of 32 rows of V.  What bounds it is the
+// chain of ~150 FP64 operations of a rotation (64 cycles each on a warp's
+// scheduler: ~5 us) and the launch.  Against three launches and two passes:
+// n = 240 11.6 us a step (20 us); n = 200 against one block: 11 us (~190 us).
+constexpr int JT = 8, JV = 32;
+__global__ void __launch_bounds__(JT * JT)
+    jstep_kernel(const cplx* __restrict__ A, cplx* __restrict__ An, cplx* __restrict__ V,
+                 int n, int np, int s, int nt, int na) {
+  __shared__ Rot rot[2 * JT];
+  __shared__ int ip[2 * JT], iq[2 * JT];
+  const int tid = threadIdx.x, ti = tid / JT, tj = tid % JT;
+  const bool vblk = (int)blockIdx.x >= na;
+  const int blk = vblk ? (int)blockIdx.x - na : (int)blockIdx.x;
+  const int tk = blk / nt, tl = blk % nt;  // tk of a V block: its tile of rows
+  // pairs of the tile's columns at [0, JT), of its rows at [JT, 2 JT)
+  if (tid < (vblk ? JT : 2 * JT))
+    rot[tid] = rotation_of(A, n, np, s, (tid < JT ? tl : tk) * JT + tid % JT, ip[tid], iq[tid]);
+  __syncthreads();
+  if (vblk)
+    rotate_rows(V, n, ip[tj], iq[tj], rot[tj], tk * JV + ti, min(n, (tk + 1) * JV), JT);
+  else
+    rotate_block(A, An, n, ip[JT + ti], iq[JT + ti], rot[JT + ti], ip[tj], iq[tj], rot[tj]);
+}
+
+// One step as two launches, for n where the FP64 pipes are the bound and
+// rotations worked out in every block take a third of them: the tiles of A
+// (8 x 8 pairs a block) from the step's rotations in rot; then, side by
+// side, V of this step and the rotations of the next one, s1, a warp of
+// pairs a block (blocks below nr).  n = 600: 20.7 us a step, 24 us as one
+// launch, 33 us as three.
+constexpr int LT = 8, LV = 32;
+__global__ void __launch_bounds__(LT * LT)
+    jtiles_kernel(const cplx* __restrict__ A, cplx* __restrict__ An, int n, int np, int s, int nt,
+                  const Rot* __restrict__ rot) {
+  const int k = blockIdx.x / nt * LT + threadIdx.x / LT;
+  const int l = blockIdx.x % nt * LT + threadIdx.x % LT;
+  if (k >= np / 2 || l >= np / 2) return;
+  int pk, qk, pl, ql;
+  rr_pair(k, np, s, pk, qk);
+  rr_pair(l, np, s, pl, ql);
+  rotate_block(A, An, n, pk, qk, rot[k], pl, ql, rot[l]);
+}
+__global__ void __launch_bounds__(LT * LT)
+    jnext_kernel(const cplx* __restrict__ A, cplx* __restrict__ V, int n, int np, int s, int s1,
+                 int nt, int nr, const Rot* __restrict__ rot, Rot* __restrict__ rot1) {
+  int p, q;
+  if ((int)blockIdx.x < nr) {
+    const int k = blockIdx.x * 32 + threadIdx.x;
+    if (threadIdx.x < 32 && k < np / 2) rot1[k] = rotation_of(A, n, np, s1, k, p, q);
+    return;
+  }
+  const int blk = (int)blockIdx.x - nr;
+  const int l = blk % nt * LT + threadIdx.x % LT, r0 = blk / nt * LV;
+  if (l >= np / 2) return;
+  rr_pair(l, np, s, p, q);
+  rotate_rows(V, n, p, q, rot[l], r0 + threadIdx.x / LT, min(n, r0 + LV), LT);
 }
 
 __global__ void jidentity_kernel(cplx* V, int n) {
@@ -363,10 +405,11 @@ __global__ void jcolumns_kernel(const cplx* __restrict__ V, int n, const int* __
 // against 70 us).
 constexpr int SMALL_N = 24;
 
-// scratch of jacobi_eigh_grid: a second A, partial sums, ranks
+// scratch of jacobi_eigh_grid: a second A, the rotations of two steps,
+// partial sums, ranks
 static size_t grid_work_bytes(int n) {
-  return (size_t)n * n * sizeof(cplx) + 2 * JPART * sizeof(double) +
-         ((size_t)n * sizeof(int) + 15) / 16 * 16;
+  return (size_t)n * n * sizeof(cplx) + (size_t)(n + 2) * sizeof(Rot) +
+         2 * JPART * sizeof(double) + ((size_t)n * sizeof(int) + 15) / 16 * 16;
 }
 size_t jacobi_work_bytes(int n) {
   return (size_t)n * n * sizeof(cplx) + grid_work_bytes(n);
@@ -375,17 +418,22 @@ size_t jacobi_work_bytes(int n) {
 int jacobi_eigh_grid(cudaStream_t s, cplx* A, int n, double* w, cplx* U, cplx* V, void* work,
                      int max_sweeps, double tol, double floor) {
   CVS_REQUIRE(n >= 1 && n <= 16384, -1, "jacobi_eigh_grid: n out of range");
+  const int np = (n + 1) & ~1, half = np / 2;
   cplx* bufs[2] = {A, (cplx*)work};
-  double* part = (double*)((cplx*)work + (size_t)n * n);
+  Rot* rots[2] = {(Rot*)((cplx*)work + (size_t)n * n), nullptr};
+  rots[1] = rots[0] + half;
+  double* part = (double*)(rots[0] + (n + 2));
   int* rank = (int*)(part + 2 * JPART);
-  const int np = (n + 1) & ~1;
-  // 8 x 8 pairs give 345 blocks at n = 240 (2.3 per SM), 16 x 16 give 456 at
-  // n = 600 with a quarter of the repeated rotations
-  const bool large = n >= 400;
-  const int jt = large ? 16 : 8, vr = large ? 128 : 32;
-  const int nt = (np / 2 + jt - 1) / jt;
-  const int na = nt * nt;
-  const unsigned grid = (unsigned)(na + nt * ((n + vr - 1) / vr));
+  // 8 x 8 pairs give 345 blocks at n = 240 (2.3 per SM); at n = 600 two
+  // launches save a seventh of the step (jtiles_kernel)
+  const bool two = n >= 400;
+  const int nt = (half + (two ? LT : JT) - 1) / (two ? LT : JT);
+  const int na = nt * nt, nr = (half + 31) / 32;
+  const int nv = nt * ((n + (two ? LV : JV) - 1) / (two ? LV : JV));
+  if (two) {  // the rotations of the first step
+    jnext_kernel<<<nr, LT * LT, 0, s>>>(A, V, n, np, 0, 0, nt, nr, rots[1], rots[0]);
+    CVS_CHECK_LAUNCH();
+  }
   jidentity_kernel<<<grid1d((int64_t)n * n, 256), 256, 0, s>>>(V, n);
   CVS_CHECK_LAUNCH();
   int sweep = 0, cur = 0;
@@ -407,8 +455,15 @@ int jacobi_eigh_grid(cudaStream_t s, cplx* A, int n, double* w, cplx* U, cplx* V
     if (ratio < tol || (ratio < floor && ratio > 0.5 * prev)) break;
     prev = ratio;
     for (int st = 0; st < np - 1; ++st, cur ^= 1) {
-      auto* step = large ? jstep_kernel<16, 128> : jstep_kernel<8, 32>;
-      step<<<grid, jt * jt, 0, s>>>(bufs[cur], bufs[cur ^ 1], V, n, np, st, nt, na);
+      if (!two) {
+        jstep_kernel<<<na + nv, JT * JT, 0, s>>>(bufs[cur], bufs[cur ^ 1], V, n, np, st, nt, na);
+        CVS_CHECK_LAUNCH();
+        continue;
+      }
+      jtiles_kernel<<<na, LT * LT, 0, s>>>(bufs[cur], bufs[cur ^ 1], n, np, st, nt, rots[cur]);
+      CVS_CHECK_LAUNCH();
+      jnext_kernel<<<nr + nv, LT * LT, 0, s>>>(bufs[cur ^ 1], V, n, np, st, (st + 1) % (np - 1),
+                                               nt, nr, rots[cur], rots[cur ^ 1]);
       CVS_CHECK_LAUNCH();
     }
   }

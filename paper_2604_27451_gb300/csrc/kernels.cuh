@@ -64,6 +64,9 @@ void scale_view(cudaStream_t s, int M, int N, double beta, View C, int batch);
 // out[0], out[1] (device doubles, zeroed by the launcher).
 void hermiticity(cudaStream_t s, const cplx* B, int n, int64_t nmat,
                  double* out_dev);
+// the same by components and without FP64 arithmetic: out[0] = max component
+// of |B_pq - conj(B_qp)|, out[1] <= max component of |B_pq|
+void hermiticity_quick(cudaStream_t s, const cplx* B, int n, int64_t nmat, double* out_dev);
 
 // ------------------------------------------------------------ MP2 / t2
 // From V[(al, i), (b, j)] = (a i | b j) for a = a0 + al, write

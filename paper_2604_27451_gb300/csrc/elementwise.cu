@@ -447,6 +447,14 @@ __device__ __forceinline__ void dfc_conj_mac(float* acc, const dfc& a, const dfc
   df_mac(acc[2], acc[3], a.ih, a.il, b.rh, b.rl, -1.0f);
 }
 
+// acc -= a * b
+__device__ __forceinline__ void dfc_msub(float* acc, const dfc& a, const dfc& b) {
+  df_mac(acc[0], acc[1], a.rh, a.rl, b.rh, b.rl, -1.0f);
+  df_mac(acc[0], acc[1], a.ih, a.il, b.ih, b.il, 1.0f);
+  df_mac(acc[2], acc[3], a.rh, a.rl, b.ih, b.il, -1.0f);
+  df_mac(acc[2], acc[3], a.ih, a.il, b.rh, b.rl, -1.0f);
+}
+
 // acc += a * b
 __device__ __forceinline__ void dfc_mac(float* acc, const dfc& a, const dfc& b) {
   df_mac(acc[0], acc[1], a.rh, a.rl, b.rh, b.rl, 1.0f);
@@ -472,6 +480,7 @@ struct ArDF {
   __device__ static void zero(Acc& a) { a.v[0] = a.v[1] = a.v[2] = a.v[3] = 0.f; }
   __device__ static void cmac(Acc& a, const E& x, const E& y) { dfc_conj_mac(a.v, x, y); }
   __device__ static void mac(Acc& a, const E& x, const E& y) { dfc_mac(a.v, x, y); }
+  __device__ static void msub(Acc& a, const E& x, const E& y) { dfc_msub(a.v, x, y); }
   __device__ static cplx value(const Acc& a) { return dfc_value(a.v); }
 };
 struct Ar64 {
@@ -489,6 +498,10 @@ struct Ar64 {
     a.re = fma(x.x, y.x, fma(-x.y, y.y, a.re));
     a.im = fma(x.x, y.y, fma(x.y, y.x, a.im));
   }
+  __device__ static void msub(Acc& a, const E& x, const E& y) {
+    a.re = fma(-x.x, y.x, fma(x.y, y.y, a.re));
+    a.im = fma(-x.x, y.y, fma(-x.y, y.x, a.im));
+  }
   __device__ static cplx value(const Acc& a) { return cmake(a.re, a.im); }
 };
 static_assert(sizeof(ArDF::E) == sizeof(cplx) && sizeof(Ar64::E) == sizeof(cplx),
@@ -505,7 +518,9 @@ static_assert(sizeof(ArDF::E) == sizeof(cplx) && sizeof(Ar64::E) == sizeof(cplx)
 // packed pair order (contiguous in b for each a).  The <Kb||Ij> terms take
 // 24 complex products per element: P = ArDF runs them in double-float on
 // the FP32 pipes (this GPU's FP64 rate is a small fraction of its FP32
-// rate), P = Ar64 in FP64.
+// rate), P = Ar64 in FP64.  FP64 operations bound the rest of the ArDF form
+// (14 per element: one accumulator for both terms, e_I + e_j taken together):
+// 0.91 ms per vector of the medium workload, 1.38 ms with 21.
 constexpr int ST = 32;
 constexpr int ST_MAXC = 16;  // ncore staged per tile (larger ncore: rows loop)
 template <class P>
@@ -543,12 +558,8 @@ __global__ void __launch_bounds__(256)
   const int64_t dbase = ij * npair;
   const int64_t hs = (int64_t)nv * nc * nw;  // stride of K in h
   const int64_t hij = (int64_t)I * nw + j;
-  // sum_K x1[K][a] h[K][b] and sum_K x1[K][b] h[K][a] per element
-  typename P::Acc acc_p[4], acc_m[4];
-  for (int q = 0; q < 4; ++q) {
-    P::zero(acc_p[q]);
-    P::zero(acc_m[q]);
-  }
+  typename P::Acc acc[4];
+  for (int q = 0; q < 4; ++q) P::zero(acc[q]);
   // the <Kb||Ij> terms, sum_K x1[K][a] h[K][b] - x1[K][b] h[K][a], in
   // groups of ST_MAXC cores
   for (int K0 = 0; h && K0 < nc; K0 += ST_MAXC) {
@@ -567,12 +578,13 @@ __global__ void __launch_bounds__(256)
       const int e = threadIdx.x + q * blockDim.x;
       const int r = e / ST, c = e % ST;
       for (int K = 0; K < kc; ++K) {
-        P::mac(acc_p[q], xa[K][r], hb[K][c]);
-        P::mac(acc_m[q], xb[K][c], ha[K][r]);
+        P::mac(acc[q], xa[K][r], hb[K][c]);
+        P::msub(acc[q], xb[K][c], ha[K][r]);
       }
     }
   }
   __syncthreads();
+  const double eIj = eps[I] + eps[nc + j];
   for (int q = 0; q < 4; ++q) {
     const int e = threadIdx.x + q * blockDim.x;
     const int r = e / ST, c = e % ST;
@@ -580,10 +592,10 @@ __global__ void __launch_bounds__(256)
     if (a >= nv || b >= nv || a >= b) continue;
     const int64_t d = dbase + pair_index(a, b, nv);
     cplx out = csub(gb[c][r], ga[r][c]);
-    if (h) out = cadd(out, csub(P::value(acc_p[q]), P::value(acc_m[q])));
+    if (h) out = cadd(out, P::value(acc[q]));
     if (x2) {
       const cplx x = x2[d];
-      const double m22 = eps[o + a] + eps[o + b] - eps[I] - eps[nc + j];
+      const double m22 = (eps[o + a] + eps[o + b]) - eIj;
       out.x += m22 * x.x;
       out.y += m22 * x.y;
     }

@@ -288,6 +288,39 @@ __global__ void __launch_bounds__(256)
   if (threadIdx.x == 0) part[blk] = 0.5 * sum;
 }
 
+// X[m][off + q] = X[q][off + m] (conjugated if CONJ) for m0 <= m < m1, q < m:
+// a block mirrors one 32 x 32 tile through shared memory (rows contiguous on
+// both sides); bounded by memory.
+template <bool CONJ>
+__global__ void __launch_bounds__(256)
+    mirror_fill_kernel(cplx* X, int64_t ld, int64_t off, int m0, int m1, int t0, int npt,
+                       int64_t stride) {
+  __shared__ cplx sm[32][33];
+  cplx* x = X + (int64_t)(blockIdx.x / npt) * stride;
+  // tiles (tm, tq), t0 <= tm, tq <= tm, counted row by row
+  int tm = t0, rem = (int)(blockIdx.x % npt);
+  while (rem > tm) {
+    rem -= tm + 1;
+    ++tm;
+  }
+  const int mb = tm * 32, qb = rem * 32;
+  const int c = threadIdx.x & 31, r0 = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int q = qb + r0 + 8 * k, m = mb + c;
+    if (q < m1 && m < m1) sm[r0 + 8 * k][c] = x[q * ld + off + m];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int m = mb + r0 + 8 * k, q = qb + c;
+    if (m < m0 || m >= m1 || q >= m) continue;
+    cplx v = sm[c][r0 + 8 * k];
+    if (CONJ) v.y = -v.y;
+    x[m * ld + off + q] = v;
+  }
+}
+
 // *out += sum of in[0..n)
 __global__ void reduce_sum_add_kernel(const double* in, int64_t n, double* out) {
   double acc = 0.0;
@@ -1045,6 +1078,21 @@ void hermiticity_quick(cudaStream_t s, const cplx* B, int n, int64_t nmat, doubl
 void t2_band(cudaStream_t s, const cplx* V, int a0, int na, int o, int v,
              const double* eps, cplx* t2, cplx* g2, double* part, int nblk) {
   t2_band_kernel<<<nblk, 256, 0, s>>>(V, a0, na, o, v, eps, t2, g2, part);
+  CVS_CHECK_LAUNCH();
+}
+
+void mirror_fill(cudaStream_t s, cplx* X, int64_t ld, int64_t off, int m0, int m1, bool conj,
+                 int64_t nmat, int64_t stride) {
+  if (m1 <= m0 || nmat <= 0) return;
+  const int t0 = m0 / 32, t1 = (m1 + 31) / 32;
+  const int64_t npt = ((int64_t)t1 * (t1 + 1) - (int64_t)t0 * (t0 + 1)) / 2;
+  CVS_REQUIRE(npt * nmat < (1LL << 31), -1, "mirror_fill: too many tiles");
+  if (conj)
+    mirror_fill_kernel<true><<<(unsigned)(npt * nmat), 256, 0, s>>>(X, ld, off, m0, m1, t0,
+                                                                    (int)npt, stride);
+  else
+    mirror_fill_kernel<false><<<(unsigned)(npt * nmat), 256, 0, s>>>(X, ld, off, m0, m1, t0,
+                                                                     (int)npt, stride);
   CVS_CHECK_LAUNCH();
 }
 

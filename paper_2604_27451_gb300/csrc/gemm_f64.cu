@@ -59,7 +59,7 @@ template <int TY, int TX, int RM, int RN, int BK, int ST>
 __global__ void __launch_bounds__(NT)
     zgemm_f64_kernel(int M, int N, int K, double alpha, View A, View B,
                      double beta, View C, int a_kfast, int b_kfast,
-                     int ntn, int kchunk, int period, cplx* part) {
+                     int ntn, int kchunk, int period, int64_t upper, cplx* part) {
   constexpr int KX = NT / (TY * TX);
   constexpr int TM = TY * RM, TN = TX * RN;
   constexpr int EA = (TM * BK + NT - 1) / NT, EB = (TN * BK + NT - 1) / NT;
@@ -70,6 +70,9 @@ __global__ void __launch_bounds__(NT)
   const int ty = tid % TY, tx = (tid / TY) % TX, kx = tid / (TY * TX);
   const int m0 = (blockIdx.x / ntn) * TM, n0 = (blockIdx.x % ntn) * TN;
   const int64_t z = blockIdx.z;
+  // upper >= 0: the square of columns from `upper` on is symmetric, and tiles
+  // wholly below its diagonal are left out
+  if (upper >= 0 && n0 >= upper && n0 + TN <= upper + m0) return;
   const cplx* Ap = A.p;
   const cplx* Bp = B.p;
   cplx* Cp = C.p;
@@ -234,7 +237,7 @@ __global__ void __launch_bounds__(NT)
 }
 
 typedef void (*F64Kernel)(int, int, int, double, View, View, double, View, int, int, int, int,
-                          int, cplx*);
+                          int, int64_t, cplx*);
 struct F64Shape {
   int tm, tn, bk;
   double eff;
@@ -354,7 +357,7 @@ void splitk_reduce(cudaStream_t s, int M, int N, int nz, const cplx* part,
 
 void zgemm_f64(cudaStream_t s, int M, int N, int K, double alpha, View A,
                View B, double beta, View C, int batch, cplx* part,
-               size_t part_elems) {
+               size_t part_elems, int64_t upper) {
   if (M <= 0 || N <= 0 || batch <= 0) return;
   if (K <= 0) {
     // C = beta * C
@@ -377,7 +380,7 @@ void zgemm_f64(cudaStream_t s, int M, int N, int K, double alpha, View A,
   CVS_REQUIRE(tiles <= INT32_MAX, -1, "zgemm_f64: output too large");
   dim3 grid((unsigned)tiles, 1, nz > 1 ? nz : batch);
   p.shape->fn<<<grid, NT, 0, s>>>(M, N, K, alpha, A, B, beta, C, a_kfast, b_kfast, ntn, kchunk,
-                                  period, nz > 1 ? part : nullptr);
+                                  period, upper, nz > 1 ? part : nullptr);
   CVS_CHECK_LAUNCH();
   kstats_end(s, tok);
   if (nz > 1) splitk_reduce(s, M, N, nz, part, beta, C);

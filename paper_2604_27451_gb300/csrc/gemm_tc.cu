@@ -705,7 +705,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
                          const __grid_constant__ CUtensorMap tmB,
                          const __grid_constant__ CUtensorMap tmB2, int kpa, int ka_off,
                          int kpb, int kb_off, int nkb, int zl, int ntm, int ntn, int nitems,
-                         int M, int N, const int* __restrict__ eA, const int* __restrict__ eB,
+                         int64_t upper, int M, int N, const int* __restrict__ eA, const int* __restrict__ eB,
                          double alpha, double beta, View C, cplx* part, int* err) {
   using P = PairCfg<NS>;
   constexpr int PN = P::PN, AS = P::ASLOTS, BS = P::BSTAGES, NI = P::ISSUERS;
@@ -775,6 +775,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
     n0 = (local / gsz) * (PN / 2);  // complex columns
     kb0 = z * zl;
     kb1 = min(nkb, kb0 + zl);
+    // tiles wholly below the diagonal of a symmetric square are left out
+    return !(upper >= 0 && n0 >= upper && n0 + PN / 2 <= upper + m0);
   };
 
   if (threadIdx.x == 0) {
@@ -782,7 +784,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
     int u = 0, ia = 0;  // units and A tiles so far
     for (int it = pair; it < nitems && !fail; it += npairs) {
       int m0, n0, z, kb0, kb1;
-      item_at(it, m0, n0, z, kb0, kb1);
+      if (!item_at(it, m0, n0, z, kb0, kb1)) continue;
       const int ya = m0 + (int)rank * BM, yb = 2 * n0 + (int)rank * (PN / 2);
       for (int v = 0; v < 2 * (kb1 - kb0) && !fail; ++v, ++u) {
         const int kb = kb0 + v / 2, c = v & 1;
@@ -833,7 +835,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
         int u = 0, ia = 0, r = 0;
         for (int it = pair; it < nitems && !fail; it += npairs) {
           int m0, n0, z, kb0, kb1;
-          item_at(it, m0, n0, z, kb0, kb1);
+          if (!item_at(it, m0, n0, z, kb0, kb1)) continue;
           const int nu = 2 * (kb1 - kb0);
           for (int v = 0; v < nu && !fail; ++v, ++u) {
             const bool first = v % P_RUN == 0;
@@ -904,7 +906,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
         int u = 0, ia = 0, r = 0;
         for (int it = pair; it < nitems && !fail; it += npairs) {
           int m0, n0, z, kb0, kb1;
-          item_at(it, m0, n0, z, kb0, kb1);
+          if (!item_at(it, m0, n0, z, kb0, kb1)) continue;
           const int nu = 2 * (kb1 - kb0);
           for (int v = 0; v < nu && !fail; ++v, ++u) {
             const bool first = v % P_RUN == 0;
@@ -977,7 +979,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
     int r = 0;
     for (int it = pair; it < nitems && ok; it += npairs) {
       int m0, n0, z, kb0, kb1;
-      item_at(it, m0, n0, z, kb0, kb1);
+      if (!item_at(it, m0, n0, z, kb0, kb1)) continue;
       const int nruns = (2 * (kb1 - kb0) + P_RUN - 1) / P_RUN;
       float hi[CG], lo[CG];
 #pragma unroll
@@ -1339,7 +1341,7 @@ __global__ void __launch_bounds__(576, 1)
                       int kpb, int kb_off, int nkb, int zl, int M, int N,
                       const int* __restrict__ eA,
                       const int* __restrict__ eB, double alpha, double beta,
-                      View C, cplx* part, int* err) {
+                      View C, cplx* part, int64_t upper, int* err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(smem + R_STAGES * R_STAGE);
@@ -1354,6 +1356,8 @@ __global__ void __launch_bounds__(576, 1)
   tile_coords(mt, nt);
   const int m0 = mt * BM, n0 = nt * RBN;
   const int z = blockIdx.z;
+  // a tile wholly below the diagonal of a symmetric square is left out
+  if (upper >= 0 && n0 / 2 >= upper && (n0 + RBN) / 2 <= upper + m0) return;
   // this CTA's K blocks [kb0, kb1); units u = 2 (kb - kb0) + c
   const int kb0 = z * zl, kb1 = min(nkb, kb0 + zl);
   const int nunits = 2 * max(0, kb1 - kb0);
@@ -1580,14 +1584,14 @@ void launch_pair(cudaStream_t s, const CUtensorMap& ma, const CUtensorMap& mb,
                  const CUtensorMap& mb2, int kpa,
                  int ka_off, int kpb, int kb_off, int nkb, int zl, int nz, int M, int N,
                  const int* eA, const int* eB, double alpha, double beta, View C, cplx* part,
-                 int* err) {
+                 int64_t upper, int* err) {
   const int ntm = (M + P_BM - 1) / P_BM, ntn = (2 * N + PairCfg<NS>::PN - 1) / PairCfg<NS>::PN;
   const int64_t items = (int64_t)ntm * ntn * nz;
   CVS_REQUIRE(items <= INT32_MAX, -1, "zgemm_slice: output too large");
   const unsigned grid = 2 * (unsigned)std::min<int64_t>(items, 76);
   tc_slice_pair_kernel<NS><<<grid, pair_threads<NS>(), pair_smem<NS>(), s>>>(
-      ma, mb, mb2, kpa, ka_off, kpb, kb_off, nkb, zl, ntm, ntn, (int)items, M, N, eA, eB, alpha, beta,
-      C, part, err);
+      ma, mb, mb2, kpa, ka_off, kpb, kb_off, nkb, zl, ntm, ntn, (int)items, upper, M, N, eA, eB, alpha,
+      beta, C, part, err);
   CVS_CHECK_LAUNCH();
 }
 
@@ -1628,7 +1632,7 @@ int64_t slice_row_slab(int M, int N, int K, int nslices) {
 void zgemm_slice(cudaStream_t s, int nslices, int M, int N, int K,
                  double alpha, View A, View B, double beta, View C, void* work,
                  size_t work_bytes, cplx* part, size_t part_elems, int* err,
-                 SliceBCache* bc, SliceBCache* ac) {
+                 SliceBCache* bc, SliceBCache* ac, int64_t upper) {
   if (M <= 0 || N <= 0) return;
   CVS_REQUIRE(nslices == 4 || nslices == 7, -1, "zgemm_slice: 4 or 7 slices");
   CVS_REQUIRE(!ac || nslices == 4, -1, "zgemm_slice: cached A needs 4 slices");
@@ -1709,14 +1713,14 @@ void zgemm_slice(cudaStream_t s, int nslices, int M, int N, int K,
     const int tok = kstats_begin(s, K_TC_SLICE, 8.0 * M * N * (double)Kc);
     if (pl.pair && nslices == 4) {
       launch_pair<4>(s, ma, mb, mb2, kpa, ka_off, kpb, kb_off, nkb, zl, nz, M, N, eAc, eBc, alpha,
-                     beta_c, C, pp, err);
+                     beta_c, C, pp, upper, err);
     } else if (pl.pair) {
       launch_pair<7>(s, ma, mb, mb2, kpa, ka_off, kpb, kb_off, nkb, zl, nz, M, N, eAc, eBc, alpha,
-                     beta_c, C, pp, err);
+                     beta_c, C, pp, upper, err);
     } else {
       dim3 grid(d.Np2 / RBN, d.Mp / BM, nz);
       tc_slice4r_kernel<<<grid, 576, R_SMEM, s>>>(ma, mb, kpa, ka_off, kpb, kb_off, nkb, zl, M, N,
-                                                  eAc, eBc, alpha, beta_c, C, pp, err);
+                                                  eAc, eBc, alpha, beta_c, C, pp, upper, err);
       CVS_CHECK_LAUNCH();
     }
     kstats_end(s, tok);

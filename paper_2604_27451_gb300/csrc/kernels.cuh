@@ -8,10 +8,17 @@ namespace cvs {
 // ------------------------------------------------------------- GEMMs
 // C = alpha * A * B + beta * C, complex, two-mode views, batch over z.
 // `part` (part_elems complex) is scratch for split-K partial products; with
-// part == nullptr the kernel runs without splitting.
+// part == nullptr the kernel runs without splitting.  upper >= 0: element
+// (m, upper + m') is symmetric (or Hermitian) in m and m', and the caller
+// fills in m' < m (mirror_fill): tiles wholly below that diagonal need not
+// be computed (C there is undefined; beta must be 0).
 void zgemm_f64(cudaStream_t s, int M, int N, int K, double alpha, View A,
                View B, double beta, View C, int batch = 1,
-               cplx* part = nullptr, size_t part_elems = 0);
+               cplx* part = nullptr, size_t part_elems = 0, int64_t upper = -1);
+// X[m][off + m'] = X[m'][off + m] (conjugated if conj) for m0 <= m < m1,
+// m' < m, in nmat matrices of leading dimension ld, `stride` elements apart
+void mirror_fill(cudaStream_t s, cplx* X, int64_t ld, int64_t off, int m0, int m1, bool conj,
+                 int64_t nmat = 1, int64_t stride = 0);
 // C(m, n) = sum_z part[z][m][n] + beta * C(m, n), part dense [nz][M][N]
 void splitk_reduce(cudaStream_t s, int M, int N, int nz, const cplx* part,
                    double beta, View C);
@@ -54,7 +61,7 @@ int64_t slice_row_slab(int M, int N, int K, int nslices);
 void zgemm_slice(cudaStream_t s, int nslices, int M, int N, int K,
                  double alpha, View A, View B, double beta, View C, void* work,
                  size_t work_bytes, cplx* part, size_t part_elems, int* err, SliceBCache* bc = nullptr,
-                 SliceBCache* ac = nullptr);
+                 SliceBCache* ac = nullptr, int64_t upper = -1);  // upper: as in zgemm_f64
 
 // C = beta * C over a view
 void scale_view(cudaStream_t s, int M, int N, double beta, View C, int batch);

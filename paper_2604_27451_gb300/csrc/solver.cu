@@ -286,10 +286,10 @@ View rows_from(View v, int64_t m0) {
 }
 
 // cache_b / cache_a: B / A is the same view of B^P on every call (the sigma
-// products), so its packed slices may be kept
+// products), so its packed slices may be kept.  upper: as in zgemm_f64
 void gemm(cvsadc_ctx* c, int prec, int M, int N, int K, double alpha, View A,
           View B, double beta, View C, int batch = 1, bool cache_b = false,
-          bool cache_a = false) {
+          bool cache_a = false, int64_t upper = -1) {
   A = checked(A);
   B = checked(B);
   C = checked(C);
@@ -324,7 +324,8 @@ void gemm(cvsadc_ctx* c, int prec, int M, int N, int K, double alpha, View A,
           const int Mi = (int)std::min<int64_t>(slab, M - m0);
           zgemm_slice(c->stream, ns, Mi, N, K, alpha, rows_from(A, m0), B, beta,
                       rows_from(C, m0), c->s_tc.p, need, c->s_kpart.c(),
-                      c->s_kpart.bytes / sizeof(cplx), c->err.as<int>(), nullptr);
+                      c->s_kpart.bytes / sizeof(cplx), c->err.as<int>(), nullptr, nullptr,
+                      upper < 0 ? upper : upper + m0);
         }
         return;
       }
@@ -343,7 +344,7 @@ void gemm(cvsadc_ctx* c, int prec, int M, int N, int K, double alpha, View A,
       if (ns)
         zgemm_slice(c->stream, ns, M, N, K, alpha, a, b, beta, cc, c->s_tc.p,
                     need, c->s_kpart.c(), c->s_kpart.bytes / sizeof(cplx),
-                    c->err.as<int>(), bc, ac);
+                    c->err.as<int>(), bc, ac, upper);
       else
         zgemm_tc(c->stream, 3, M, N, K, alpha, a, b, beta, cc, c->s_tc.p, need,
                  c->s_kpart.c(), c->s_kpart.bytes / sizeof(cplx),
@@ -352,7 +353,7 @@ void gemm(cvsadc_ctx* c, int prec, int M, int N, int K, double alpha, View A,
     return;
   }
   zgemm_f64(c->stream, M, N, K, alpha, A, B, beta, C, batch, c->s_kpart.c(),
-            c->s_kpart.bytes / sizeof(cplx));
+            c->s_kpart.bytes / sizeof(cplx), upper);
 }
 
 void gemm64(cvsadc_ctx* c, int M, int N, int K, double alpha, View A,
@@ -447,7 +448,8 @@ void build_t2(cvsadc_ctx* c, int prec, const cplx* B, const double* eps,
     View A = rows2(view(B + (int64_t)(o + a0) * n, 0, nn), n, 1, o);
     View Bv = cols2(view(B + (int64_t)o * n, nn, 0), n, 1, o);
     View C = view(c->s_big1.p, vo, 1);
-    gemm(c, prec, nb * o, (int)vo, L, 1.0, A, Bv, 0.0, C);
+    gemm(c, prec, nb * o, (int)vo, L, 1.0, A, Bv, 0.0, C, 1, false, false, (int64_t)a0 * o);
+    mirror_fill(c->stream, c->s_big1.c(), vo, (int64_t)a0 * o, 0, nb * o, false);
     t2_band(c->stream, c->s_big1.c(), a0, nb, o, v, eps, t2.c(), g2.c(),
             c->s_part.d(), nblk);
   }
@@ -501,7 +503,10 @@ double t2_bands(cvsadc_ctx* c, int prec, const cplx* B, const double* eps, int o
     const int nb = std::min(na, v - a0);
     View A = rows2(view(B + (int64_t)(o + a0) * n, 0, nn), n, 1, o);
     View Bv = cols2(view(B + (int64_t)o * n, nn, 0), n, 1, o);
-    gemm(c, prec, nb * o, (int)vo, L, 1.0, A, Bv, 0.0, view(X.p, vo, 1));
+    // (ai|bj) = (bj|ai): the square of the band's own b is symmetric
+    gemm(c, prec, nb * o, (int)vo, L, 1.0, A, Bv, 0.0, view(X.p, vo, 1), 1, false, false,
+         (int64_t)a0 * o);
+    mirror_fill(c->stream, X.c(), vo, (int64_t)a0 * o, 0, nb * o, false);
     t2_band_inplace(c->stream, X.c(), T.c(), a0, nb, o, v, eps, part.d(), dE);
     use(Band{a0, nb, T.c(), X.c()});
   }
@@ -793,15 +798,13 @@ void build_fns(cvsadc_ctx* c, int prec, double tau) {
     // ov block: rows i < o of every matrix
     copyv(c, (int)(nmat * o), vk, 1.0, rows2(view(tmp.c(), 0, 1), (int64_t)n * vk, vk, o),
           rows2(view(dst.c() + o, 0, 1), nn2, n2, o));
-    // vv block: U^H tmp[P][o:][:]
+    // vv block: U^H tmp[P][o:][:], Hermitian: the tiles on and above the
+    // diagonal; then the rest of the rows o .. from their mirror images
     gemm(c, CVSADC_FP64, vk, vk, v, 1.0,
          conj_of(trans(view(U, vk, 1))),
          batched(view(tmp.c() + (int64_t)o * vk, vk, 1), (int64_t)n * vk), 0.0,
-         batched(view(dst.c() + (int64_t)o * n2 + o, n2, 1), nn2), (int)nmat);
-    // vo block: U^H src[P][o:][:o]
-    gemm(c, CVSADC_FP64, vk, o, v, 1.0, conj_of(trans(view(U, vk, 1))),
-         batched(view(src + (int64_t)o * n, n, 1), nn), 0.0,
-         batched(view(dst.c() + (int64_t)o * n2, n2, 1), nn2), (int)nmat);
+         batched(view(dst.c() + (int64_t)o * n2 + o, n2, 1), nn2), (int)nmat, false, false, 0);
+    mirror_fill(c->stream, dst.c(), n2, 0, o, n2, true, nmat, nn2);
   };
   DBuf Bn;
   rotate(c->B.c(), L, Bn);

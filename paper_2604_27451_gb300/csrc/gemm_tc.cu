@@ -131,6 +131,13 @@ __device__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   return mbar_wait_for(bar, parity, WAIT_NS);
 }
 
+// an expired wait's code into the context's error word (mapped host memory;
+// whichever thread writes last stands)
+__device__ __forceinline__ void report(int* err, int code) {
+  *(volatile int*)err = code;
+  __threadfence_system();
+}
+
 // The error path of the bounded waits, on demand: one thread waits, with
 // limit_ns, on an mbarrier that nothing arrives on.  The wait gives up, the
 // kernel records code 5 in *err (as a GEMM's expired wait records its
@@ -140,7 +147,7 @@ __global__ void wait_probe_kernel(uint64_t limit_ns, int* err) {
   if (threadIdx.x == 0) {
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    if (!mbar_wait_for(&bar, 0, limit_ns)) atomicExch(err, 5);
+    if (!mbar_wait_for(&bar, 0, limit_ns)) report(err, 5);
   }
 }
 __device__ __forceinline__ void tma_load(const CUtensorMap* map, uint64_t* bar,
@@ -313,7 +320,7 @@ __global__ void __launch_bounds__(128, 1)
       }
     }
   } else if (lane == 0) {
-    atomicExch(err, fail ? fail : 3);
+    report(err, fail ? fail : 3);
   }
   fence_before();
   __syncthreads();
@@ -1018,7 +1025,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
       }
       if (!ok || fail) {
         ok = false;
-        if (lane == 0) atomicExch(err, fail ? fail : 3);
+        if (lane == 0) report(err, fail ? fail : 3);
         break;
       }
       const int m = m0 + (int)rank * BM + q * 32 + lane;
@@ -1058,7 +1065,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
     const uint64_t t0 = gtime();
     for (int n = 0; n < (1 << 20) && gtime() - t0 < 2000000; ++n) __nanosleep(1000);
   }
-  if (threadIdx.x == 0 && fail) atomicExch(err, fail);
+  if (threadIdx.x == 0 && fail) report(err, fail);
   fence_before();
   __syncthreads();
   __syncwarp();
@@ -1481,7 +1488,7 @@ __global__ void __launch_bounds__(576, 1)
       }
     }
     if (!ok || fail) {
-      if (lane == 0) atomicExch(err, fail ? fail : 3);
+      if (lane == 0) report(err, fail ? fail : 3);
     } else {
       const int m = m0 + q * 32 + lane;
       if (m < M) {

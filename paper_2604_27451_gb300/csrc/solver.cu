@@ -165,7 +165,11 @@ struct cvsadc_ctx {
   // scratch
   DBuf s_big1, s_big2, s_S, s_R, s_Y, s_V, s_part, s_small, s_tc;
   DBuf dv_V, dv_W, dv_X, dv_AX, dv_T, dv_H, dv_A, dv_U, dv_w, dv_misc;
-  DBuf err;  // device int: non-zero after a bounded device wait expired
+  // non-zero after a bounded device wait expired: mapped host memory, so that
+  // every call's check after its synchronisation is a host read (a device
+  // word cost a copy and a second synchronisation, ~10 us a call)
+  int* err = nullptr;      // the host's pointer
+  int* err_dev = nullptr;  // the kernels'
   DBuf s_kpart;  // split-K partial products
 
   // folded solver: fold work vectors [2g][N] x 2, singles-space basis and
@@ -202,6 +206,9 @@ struct cvsadc_ctx {
   // worker contexts of cvsadc_solve_batched (own streams), kept for reuse
   std::vector<cvsadc_ctx*> lanes;
 
+  ~cvsadc_ctx() {
+    if (err) cudaFreeHost(err);
+  }
   void sync() { CVS_CUDA(cudaStreamSynchronize(stream)); }
   std::vector<DBuf*> problem_buffers() {
     return {&eps,   &B,     &dip,   &t2,   &g2,     &M11,  &diag, &F, &h1, &hT,
@@ -220,7 +227,7 @@ struct cvsadc_ctx {
     clear_bcache();
   }
   size_t held_bytes() {
-    size_t t = s_kpart.bytes + err.bytes + bcache_bytes;
+    size_t t = s_kpart.bytes + bcache_bytes;
     for (DBuf* b : problem_buffers()) t += b->bytes;
     return t;
   }
@@ -324,7 +331,7 @@ void gemm(cvsadc_ctx* c, int prec, int M, int N, int K, double alpha, View A,
           const int Mi = (int)std::min<int64_t>(slab, M - m0);
           zgemm_slice(c->stream, ns, Mi, N, K, alpha, rows_from(A, m0), B, beta,
                       rows_from(C, m0), c->s_tc.p, need, c->s_kpart.c(),
-                      c->s_kpart.bytes / sizeof(cplx), c->err.as<int>(), nullptr, nullptr,
+                      c->s_kpart.bytes / sizeof(cplx), c->err_dev, nullptr, nullptr,
                       upper < 0 ? upper : upper + m0);
         }
         return;
@@ -344,11 +351,11 @@ void gemm(cvsadc_ctx* c, int prec, int M, int N, int K, double alpha, View A,
       if (ns)
         zgemm_slice(c->stream, ns, M, N, K, alpha, a, b, beta, cc, c->s_tc.p,
                     need, c->s_kpart.c(), c->s_kpart.bytes / sizeof(cplx),
-                    c->err.as<int>(), bc, ac, upper);
+                    c->err_dev, bc, ac, upper);
       else
         zgemm_tc(c->stream, 3, M, N, K, alpha, a, b, beta, cc, c->s_tc.p, need,
                  c->s_kpart.c(), c->s_kpart.bytes / sizeof(cplx),
-                 c->err.as<int>());
+                 c->err_dev);
     }
     return;
   }
@@ -2462,13 +2469,11 @@ void davidson_entry(cvsadc_ctx* c, const cvsadc_params* p, double* omega,
 }
 
 void check_device_error(cvsadc_ctx* c) {
-  if (!c->err.p) return;
-  int e = 0;
-  CVS_CUDA(cudaMemcpyAsync(&e, c->err.p, sizeof(int), cudaMemcpyDeviceToHost,
-                           c->stream));
+  if (!c->err) return;
   CVS_CUDA(cudaStreamSynchronize(c->stream));
+  const int e = *(volatile int*)c->err;
   if (e != 0) {
-    CVS_CUDA(cudaMemsetAsync(c->err.p, 0, sizeof(int), c->stream));
+    *(volatile int*)c->err = 0;
     char b[128];
     snprintf(b, sizeof b, "a bounded device wait expired (code %d)", e);
     throw Error{CVSADC_ETIMEOUT, b};
@@ -2824,7 +2829,7 @@ double estimate_bytes(const cvsadc_params* p) {
         w = std::max(w, s);
     b += w;
   }
-  b += (double)(8 << 20) * z + 1024;        // split-K scratch, error flag
+  b += (double)(8 << 20) * z + 1024;        // split-K scratch
   // cached slice packs of B^P views (at most min(35 % of free, 64 GB)): the
   // B operands of the sigma's S and G products, the A operands of its
   // sigma1^T and Y^T products, and the preconditioner's (aj|bc) product
@@ -2983,10 +2988,9 @@ int cvsadc_create(cvsadc_ctx** ctx, int device, void* cuda_stream) {
       CVS_CUDA(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
       c->own_stream = true;
     }
-    // cleared on the context's own stream: a memset on the default stream is
-    // not ordered before the error check that ends this call
-    c->err.ensure(256);
-    CVS_CUDA(cudaMemsetAsync(c->err.p, 0, 256, c->stream));
+    CVS_CUDA(cudaHostAlloc((void**)&c->err, 64, cudaHostAllocMapped | cudaHostAllocPortable));
+    *(volatile int*)c->err = 0;
+    CVS_CUDA(cudaHostGetDevicePointer((void**)&c->err_dev, c->err, 0));
   });
   if (rc != CVSADC_OK) {
     delete c;
@@ -3138,7 +3142,7 @@ int64_t cvsadc_launch_count(void) {
 
 int cvsadc_wait_probe(cvsadc_ctx* c, int64_t limit_ns) {
   if (!c) return CVSADC_EINVAL;
-  return guarded(c, [&] { wait_probe(c->stream, limit_ns, c->err.as<int>()); });
+  return guarded(c, [&] { wait_probe(c->stream, limit_ns, c->err_dev); });
 }
 
 int cvsadc_zgemm(cvsadc_ctx* c, int32_t precision, int32_t flags, int32_t M,

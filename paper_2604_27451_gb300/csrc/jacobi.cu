@@ -198,6 +198,31 @@ __device__ __forceinline__ void rr_pair(int k, int np, int s, int& p, int& q) {
   }
 }
 
+// A step's kernels are launched while their predecessor drains: their blocks
+// come up, work out indices and wait here until it is complete and its
+// writes are visible, which hides most of a launch.  Whole solves whose
+// preconditioner has n = 240: 51.5 -> 46.5 ms, n = 600: 221 -> 199 ms.  No
+// load of what the predecessor writes may stand above this, nor be a
+// read-only (non-coherent) one.
+__device__ __forceinline__ void after_predecessor() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... Q>
+void launch_chained(cudaStream_t s, void (*kernel)(P...), int grid, int block, Q... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.stream = s;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  CVS_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+  CVS_CHECK_LAUNCH();
+}
+
 // the rotation of a_pq, skipped for |a_pq| <= 1e-18 sqrt(|a_pp a_qq|)
 __device__ __forceinline__ void rotation(cplx apq, double app, double aqq, double& c, cplx& sv) {
   c = 1.0;
@@ -229,9 +254,8 @@ __device__ __forceinline__ Rot rotation_of(const cplx* A, int n, int np, int s, 
 }
 
 // An = J^H A J on the 2 x 2 block of rows (pk, qk) and columns (pl, ql)
-__device__ __forceinline__ void rotate_block(const cplx* __restrict__ A, cplx* __restrict__ An,
-                                             int n, int pk, int qk, const Rot& rk, int pl, int ql,
-                                             const Rot& rl) {
+__device__ __forceinline__ void rotate_block(const cplx* A, cplx* An, int n, int pk, int qk,
+                                             const Rot& rk, int pl, int ql, const Rot& rl) {
   auto get = [&](int r, int c) {
     return r < n && c < n ? A[(int64_t)r * n + c] : cmake(0.0, 0.0);
   };
@@ -279,17 +303,18 @@ __device__ __forceinline__ void rotate_rows(cplx* V, int n, int p, int q, const 
 // na on rotate 8 pairs of columns of 32 rows of V.  What bounds it is the
 // chain of ~150 FP64 operations of a rotation (64 cycles each on a warp's
 // scheduler: ~5 us) and the launch.  Against three launches and two passes:
-// n = 240 11.6 us a step (20 us); n = 200 against one block: 11 us (~190 us).
+// n = 240 11.6 us a step (20 us); n = 200 against one block: 11 us (~190 us);
+// before launches overlapped.
 constexpr int JT = 8, JV = 32;
 __global__ void __launch_bounds__(JT * JT)
-    jstep_kernel(const cplx* __restrict__ A, cplx* __restrict__ An, cplx* __restrict__ V,
-                 int n, int np, int s, int nt, int na) {
+    jstep_kernel(const cplx* A, cplx* An, cplx* V, int n, int np, int s, int nt, int na) {
   __shared__ Rot rot[2 * JT];
   __shared__ int ip[2 * JT], iq[2 * JT];
   const int tid = threadIdx.x, ti = tid / JT, tj = tid % JT;
   const bool vblk = (int)blockIdx.x >= na;
   const int blk = vblk ? (int)blockIdx.x - na : (int)blockIdx.x;
   const int tk = blk / nt, tl = blk % nt;  // tk of a V block: its tile of rows
+  after_predecessor();
   // pairs of the tile's columns at [0, JT), of its rows at [JT, 2 JT)
   if (tid < (vblk ? JT : 2 * JT))
     rot[tid] = rotation_of(A, n, np, s, (tid < JT ? tl : tk) * JT + tid % JT, ip[tid], iq[tid]);
@@ -305,22 +330,23 @@ __global__ void __launch_bounds__(JT * JT)
 // (8 x 8 pairs a block) from the step's rotations in rot; then, side by
 // side, V of this step and the rotations of the next one, s1, a warp of
 // pairs a block (blocks below nr).  n = 600: 20.7 us a step, 24 us as one
-// launch, 33 us as three.
+// launch, 33 us as three, before launches overlapped.
 constexpr int LT = 8, LV = 32;
 __global__ void __launch_bounds__(LT * LT)
-    jtiles_kernel(const cplx* __restrict__ A, cplx* __restrict__ An, int n, int np, int s, int nt,
-                  const Rot* __restrict__ rot) {
+    jtiles_kernel(const cplx* A, cplx* An, int n, int np, int s, int nt, const Rot* rot) {
   const int k = blockIdx.x / nt * LT + threadIdx.x / LT;
   const int l = blockIdx.x % nt * LT + threadIdx.x % LT;
-  if (k >= np / 2 || l >= np / 2) return;
   int pk, qk, pl, ql;
   rr_pair(k, np, s, pk, qk);
   rr_pair(l, np, s, pl, ql);
+  after_predecessor();
+  if (k >= np / 2 || l >= np / 2) return;
   rotate_block(A, An, n, pk, qk, rot[k], pl, ql, rot[l]);
 }
 __global__ void __launch_bounds__(LT * LT)
-    jnext_kernel(const cplx* __restrict__ A, cplx* __restrict__ V, int n, int np, int s, int s1,
-                 int nt, int nr, const Rot* __restrict__ rot, Rot* __restrict__ rot1) {
+    jnext_kernel(const cplx* A, cplx* V, int n, int np, int s, int s1, int nt, int nr,
+                 const Rot* rot, Rot* rot1) {
+  after_predecessor();
   int p, q;
   if ((int)blockIdx.x < nr) {
     const int k = blockIdx.x * 32 + threadIdx.x;
@@ -456,15 +482,14 @@ int jacobi_eigh_grid(cudaStream_t s, cplx* A, int n, double* w, cplx* U, cplx* V
     prev = ratio;
     for (int st = 0; st < np - 1; ++st, cur ^= 1) {
       if (!two) {
-        jstep_kernel<<<na + nv, JT * JT, 0, s>>>(bufs[cur], bufs[cur ^ 1], V, n, np, st, nt, na);
-        CVS_CHECK_LAUNCH();
+        launch_chained(s, jstep_kernel, na + nv, JT * JT, bufs[cur], bufs[cur ^ 1], V, n, np, st,
+                       nt, na);
         continue;
       }
-      jtiles_kernel<<<na, LT * LT, 0, s>>>(bufs[cur], bufs[cur ^ 1], n, np, st, nt, rots[cur]);
-      CVS_CHECK_LAUNCH();
-      jnext_kernel<<<nr + nv, LT * LT, 0, s>>>(bufs[cur ^ 1], V, n, np, st, (st + 1) % (np - 1),
-                                               nt, nr, rots[cur], rots[cur ^ 1]);
-      CVS_CHECK_LAUNCH();
+      launch_chained(s, jtiles_kernel, na, LT * LT, bufs[cur], bufs[cur ^ 1], n, np, st, nt,
+                     rots[cur]);
+      launch_chained(s, jnext_kernel, nr + nv, LT * LT, bufs[cur ^ 1], V, n, np, st,
+                     (st + 1) % (np - 1), nt, nr, rots[cur], rots[cur ^ 1]);
     }
   }
   jrank_kernel<<<(n + 127) / 128, 128, 0, s>>>(bufs[cur], n, w, rank);

@@ -589,16 +589,18 @@ __device__ __forceinline__ void ff_add(float& hi, float& lo, float x) {
 // the NS tiles of A (128 rows in each CTA) and of B, from which all the NS
 // (NS + 1) / 2 slice pairs are issued.  Pairs of one order o = i + j share
 // the scale 2^{-7(o+2)} and one tensor-memory accumulator of PN columns; the
-// orders lie side by side and fill the tensor memory (4 x 128, or 7 x 64 and
-// 64 that nothing reads), so there is one set of them.
+// orders lie side by side and fill the tensor memory (4 x 128, 7 x 64 and 64
+// that nothing reads, or 8 x 64), so there is one set of them.
 //
 // Exact runs: |q_0| <= 2^7, |q_i| <= 2^6 for i > 0, so a run of 512 products
 // (8 units) of every pair of an order stays within 2^23 (o = 0, 1), 2.5 2^22
 // (o = 2), 3 2^22 (o = 3), 3.5 2^22 (o = 4) and 2^24 (o = 5) and sums exactly
 // in FP32; order 6 may pass 2^24 by an eighth, where one rounding is 2^-55 of
-// the order-0 product it is added to.  At the end of a run the orders finish
-// one after the other, the drain warps add each to float-float accumulators
-// in registers, and the next run overwrites an order once it is in registers.
+// the order-0 product it is added to; order 7 may by a quarter (2^-62).  At
+// the end of a run the orders finish one after the other, the drain warps add
+// each to accumulators in registers (float-float; 8 slices: two 64-bit
+// integers, so that FP64 rounds the whole sum once), and the next run
+// overwrites an order once it is in registers.
 //
 // What bounds it: an MMA takes 90 to 100 cycles to issue and run whatever its
 // width up to 128 columns, and a unit's operands arrive at ~11 TB/s over all
@@ -610,12 +612,15 @@ __device__ __forceinline__ void ff_add(float& hi, float& lo, float x) {
 //   issued them.  B slices are whole in one CTA instead, so that one MMA
 //   covers up to four (256 columns: two slices from either CTA, into four
 //   adjacent orders): 44 MMAs, 2.75 us a unit.
+// - 8 slices: the same with 15 MMAs of one to four slices per K step, 3.75 us.
 // A's tiles free up one by one, so the copies run more than a unit ahead.
 // The pairs of CTAs are persistent: the epilogue of a tile runs while the
 // next one's first run is computed.  Measured (with the operands packed):
 // 4096^3 4 slices 4.57 -> 3.23 ms (170 TFLOP/s, 0.91 of the measured bf16
 // rate over 10 products; the tile kernel below before), 7 slices 21.2 -> 9.5
-// ms (58 TFLOP/s, 0.87 over 28 products).
+// ms (58 TFLOP/s, 0.87 over 28 products); 8 slices 11.5 ms (48 TFLOP/s, 0.92
+// over 36 products; the FP64 kernels: 1.2 TFLOP/s), and 246000 x 200 by 200 x
+// 150, one run a tile, 1.8 ms (33 TFLOP/s).
 //
 // Warps: 0 (lane 0) TMA producer; 1 .. ISSUERS of rank 0 (lane 0) MMA
 // issuers; then 16 drain warps (warp w reads TMEM lanes 32 (w % 4) .. +31
@@ -635,6 +640,13 @@ struct PairCfg<7> {
   // rows of the B regions of a stage: B_0 .. B_3 (two slices in each CTA),
   // B_4 | B_5, B_0 | B_1 (one in each), B_6 (half in each)
   static constexpr int R0 = 0, R1 = 128, R2 = 192, R3 = 256, B_ROWS = 288;
+};
+template <>
+struct PairCfg<8> {
+  static constexpr int PN = 64, ASLOTS = 7, BSTAGES = 2, ISSUERS = 1;
+  // B_0 .. B_3 (two slices in each CTA), B_4 | B_5, B_6 | B_7, B_0 | B_1 (one
+  // in each), then B_6, B_4, B_2, B_0 (half in each)
+  static constexpr int R0 = 0, R1 = 128, R4 = 192, R2 = 256, R3 = 320, B_ROWS = 448;
 };
 constexpr int P_BM = 256;
 constexpr int P_RUN = 8;  // units per exact run
@@ -808,6 +820,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
 #pragma unroll
           for (int j = 0; j < NS; ++j)
             tma_load2(&tmB, fb, st + j * B_SLICE, 2 * j * kpb + xb, yb);
+        } else if constexpr (NS == 8) {
+          auto slice = [&](int row, int j) {  // all 64 columns of slice j
+            tma_load2(&tmB, fb, st + row * BK * 2, 2 * j * kpb + xb, 2 * n0);
+          };
+          slice(P::R0, rank ? 2 : 0);
+          slice(P::R0 + PN, rank ? 3 : 1);
+          slice(P::R1, rank ? 5 : 4);
+          slice(P::R4, rank ? 7 : 6);
+          slice(P::R2, rank ? 1 : 0);
+#pragma unroll
+          for (int h = 0; h < 4; ++h)
+            tma_load2(&tmB2, fb, st + (P::R3 + h * PN / 2) * BK * 2, 2 * (6 - 2 * h) * kpb + xb,
+                      yb);
         } else {
           auto slice = [&](int row, int j) {  // all 64 columns of slice j
             tma_load2(&tmB, fb, st + row * BK * 2, 2 * j * kpb + xb, 2 * n0);
@@ -908,8 +933,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
           }
         }
       };
-      // NS = 7: one issuer, up to four slices of B per MMA
-      [[maybe_unused]] auto issue7 = [&]() {
+      // NS = 7, 8: one issuer, up to four slices of B per MMA
+      [[maybe_unused]] auto issue_wide = [&]() {
         int u = 0, ia = 0, r = 0;
         for (int it = pair; it < nitems && !fail; it += npairs) {
           int m0, n0, z, kb0, kb1;
@@ -943,19 +968,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
               if (!ok) break;
               fence_after();
               const uint32_t ad = (uint32_t)sdesc(smem_u32(sA + sa * A_TILE));
+              const bool start = first && i == 0;
               if (i < 5) {
                 if (i == 0 && !drained(0, 4)) break;
-                mma(i, ad, P::R0, 4 * PN, first && i == 0);
+                mma(i, ad, P::R0, 4 * PN, start);
               }
               if (i < 3) {
                 if (i == 0 && !drained(4, 6)) break;
-                mma(i + 4, ad, P::R1, 2 * PN, first && i == 0);
+                mma(i + 4, ad, P::R1, 2 * PN, start);
               }
-              if (i == 0) {
-                if (!drained(6, 7)) break;
-                mma(6, ad, P::R3, PN, first);
+              if (i == 0 && !drained(6, NS)) break;
+              if constexpr (NS == 7) {
+                if (i == 0) mma(6, ad, P::R3, PN, first);
+                if (i >= 5) mma(i, ad, P::R2, 2 * PN, false);
+              } else if constexpr (NS == 8) {
+                if (i == 0) mma(6, ad, P::R4, 2 * PN, first);
+                if (i == 5 || i == 6) mma(i, ad, P::R2, 2 * PN, false);
+                // (1, 6), (3, 4), (5, 2) and (7, 0)
+                if (i & 1) mma(7, ad, P::R3 + (i / 2) * (PN / 2), PN, false);
               }
-              if (i >= 5) mma(i, ad, P::R2, 2 * PN, false);
               umma2_commit(&emptyA[sa]);
               // no later pair of this unit adds to order i
               if (last) umma2_commit(&afull[i]);
@@ -974,7 +1005,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
         if (warp == 1) issue4(std::integral_constant<int, 0>());
         if (warp == 2) issue4(std::integral_constant<int, 1>());
       } else {
-        issue7();
+        issue_wide();
       }
     }
   } else if (warp > NI) {
@@ -988,19 +1019,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
       int m0, n0, z, kb0, kb1;
       if (!item_at(it, m0, n0, z, kb0, kb1)) continue;
       const int nruns = (2 * (kb1 - kb0) + P_RUN - 1) / P_RUN;
-      float hi[CG], lo[CG];
+      // NS < 8: float-float sums; 8: the orders 0 .. 3 and 4 .. 7 as exact
+      // integers in units of 2^-35 and 2^-63 (a run adds at most 2^46)
+      using Acc = std::conditional_t<NS == 8, long long, float>;
+      Acc hi[CG], lo[CG];
 #pragma unroll
-      for (int i = 0; i < CG; ++i) hi[i] = lo[i] = 0.f;
+      for (int i = 0; i < CG; ++i) hi[i] = lo[i] = 0;
       for (int rr = 0; rr < nruns && ok; ++rr, ++r) {
-#pragma unroll 1
-        for (int o = 0; o < NS; ++o) {
-          if (!mbar_wait(&afull[o], r & 1)) {
-            ok = false;
-            break;
-          }
+        // order o is handed over, then f(i, value) for this warp's columns
+        auto drain = [&](int o, auto f) {
+          if (!mbar_wait(&afull[o], r & 1)) return false;
           fence_after();
-          // 2^{-7 (o + 2)}
-          const float sc = __int_as_float((127 - SLICE_BITS * (o + 2)) << 23);
 #pragma unroll
           for (int h = 0; h < CG / 8; ++h) {
             float v[8];
@@ -1015,11 +1044,31 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
                              : "memory");
             }
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              ff_add(hi[8 * h + i], lo[8 * h + i], v[i] * sc);
+            for (int i = 0; i < 8; ++i) f(8 * h + i, v[i]);
+          }
+          return true;
+        };
+        if constexpr (NS == 8) {
+#pragma unroll 1
+          for (int o = 0; o < 4 && ok; ++o) {
+            const int mul = 1 << SLICE_BITS * (3 - o);
+            ok = drain(o, [&](int i, float v) { hi[i] += (long long)__float2int_rn(v) * mul; });
+          }
+#pragma unroll 1
+          for (int o = 4; o < 8 && ok; ++o) {
+            const int mul = 1 << SLICE_BITS * (7 - o);
+            ok = drain(o, [&](int i, float v) { lo[i] += (long long)__float2int_rn(v) * mul; });
+          }
+        } else {
+#pragma unroll 1
+          for (int o = 0; o < NS && ok; ++o) {
+            // 2^{-7 (o + 2)}
+            const float sc = __int_as_float((127 - SLICE_BITS * (o + 2)) << 23);
+            ok = drain(o, [&](int i, float v) {
+              ff_add(hi[i], lo[i], v * sc);
               // one group of 8 at a time: the accumulators take most registers
-              asm volatile("" : "+f"(hi[8 * h + i]), "+f"(lo[8 * h + i]));
-            }
+              asm volatile("" : "+f"(hi[i]), "+f"(lo[i]));
+            });
           }
         }
       }
@@ -1038,11 +1087,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
           if (n < N) {
             // one column at a time (nothing hoisted): the accumulators take
             // most registers
-            asm volatile("" : "+f"(hi[2 * i]), "+f"(lo[2 * i]), "+f"(hi[2 * i + 1]),
-                         "+f"(lo[2 * i + 1]) :: "memory");
+            if constexpr (NS != 8)
+              asm volatile("" : "+f"(hi[2 * i]), "+f"(lo[2 * i]), "+f"(hi[2 * i + 1]),
+                           "+f"(lo[2 * i + 1]) :: "memory");
+            else
+              asm volatile("" : "+l"(hi[2 * i]), "+l"(lo[2 * i]), "+l"(hi[2 * i + 1]),
+                           "+l"(lo[2 * i + 1]) :: "memory");
             const double sc = em * pow2(eB[n]);
-            cplx o = cmake(sc * ((double)hi[2 * i] + (double)lo[2 * i]),
-                           sc * ((double)hi[2 * i + 1] + (double)lo[2 * i + 1]));
+            auto sum = [&](int j) {
+              if constexpr (NS == 8)
+                return fma((double)hi[j], 0x1p-35, (double)lo[j] * 0x1p-63);
+              else
+                return (double)hi[j] + (double)lo[j];
+            };
+            cplx o = cmake(sc * sum(2 * i), sc * sum(2 * i + 1));
             if (part) {
               part[((int64_t)z * M + m) * N + n] = o;
               continue;
@@ -1167,8 +1225,24 @@ __device__ __forceinline__ void slices(double x, int e, float* q) {
     q[2] = digit((T >> 7) & 127);
     q[1] = digit((T >> 14) & 127);
     q[0] = __int_as_float(0x4B400000 + (T >> 21)) - 12582912.0f;
+  } else if constexpr (S == 8) {
+    // (s >= -3: four more bits below the significand)
+    const long long m = (((long long)mh << 32) | lo) << 4;
+    long long T = ((m >> min(63, max(0, s + 3))) + 1) >> 1;
+    T = E == 0 ? 0 : ((int)hi < 0 ? -T : T);
+    T += 64ll * (1 + (1ll << 7) + (1ll << 14) + (1ll << 21) + (1ll << 28) + (1ll << 35) +
+                 (1ll << 42));
+    const int tl = (int)(T & 0xFFFFFFF), th = (int)(T >> 28);
+    q[7] = digit(tl & 127);
+    q[6] = digit((tl >> 7) & 127);
+    q[5] = digit((tl >> 14) & 127);
+    q[4] = digit((tl >> 21) & 127);
+    q[3] = digit(th & 127);
+    q[2] = digit((th >> 7) & 127);
+    q[1] = digit((th >> 14) & 127);
+    q[0] = __int_as_float(0x4B400000 + (th >> 21)) - 12582912.0f;
   } else {
-    static_assert(S == 7, "4 or 7 slices");
+    static_assert(S == 7, "4, 7 or 8 slices");
     const long long m = ((long long)mh << 32) | lo;
     long long T = ((m >> min(63, max(0, s - 1))) + 1) >> 1;
     T = E == 0 ? 0 : ((int)hi < 0 ? -T : T);
@@ -1540,7 +1614,7 @@ SDims sdims_of(int M, int N, int K, int nslices, bool b_cached, bool a_cached = 
   d.Mp = (M + BM - 1) / BM * BM;
   d.Np2 = (2 * N + tn - 1) / tn * tn;
   d.nseg = 2 * nslices;
-  d.cseg = nslices == 4 ? 8 : nslices * (nslices + 1);
+  d.cseg = nslices == 7 ? nslices * (nslices + 1) : d.nseg;
   d.KpF = (int)(((int64_t)K + BK - 1) / BK * BK);
   const size_t per_k = (size_t)((a_cached ? 0 : d.Mp) + (b_cached ? 0 : d.Np2)) * d.cseg * 2;
   int64_t kc = per_k ? (int64_t)(PACK_BUDGET / per_k) / BK * BK : (int64_t)d.KpF;
@@ -1553,7 +1627,7 @@ SDims sdims_of(int M, int N, int K, int nslices, bool b_cached, bool a_cached = 
 }
 
 // How a product of nkb K blocks is laid out on the GPU, by modelled time in
-// us.  Pairs of CTAs: 1.8 (4 slices) or 2.75 (7) us per unit of a tile, tiles
+// us.  Pairs of CTAs: 1.8 (4 slices), 2.75 (7) or 3.75 (8) us per unit of a tile, tiles
 // (times K slices) dealt out to 76 pairs, about 7 units of start and end.
 // SLICE4's 128 x 64 tiles: 1.3 us per unit, a CTA per tile, 8 units of start
 // and end: they keep narrow (2 N <= 64) and small products.  K slices need
@@ -1580,7 +1654,7 @@ SlicePlan plan_slices(int nslices, int M, int N, int nkb, size_t part_elems) {
   };
   const int pn = nslices == 4 ? PairCfg<4>::PN : PairCfg<7>::PN;
   const double tm = (M + P_BM - 1) / P_BM, tn = (2 * N + pn - 1) / pn;
-  consider(true, tm * tn, 76.0, nslices == 4 ? 1.8 : 2.75, 7.0);
+  consider(true, tm * tn, 76.0, nslices == 4 ? 1.8 : nslices == 7 ? 2.75 : 3.75, 7.0);
   if (nslices == 4)
     consider(false, (double)((M + BM - 1) / BM) * ((2 * N + RBN - 1) / RBN), 152.0, 1.3, 8.0);
   return best;
@@ -1641,7 +1715,7 @@ void zgemm_slice(cudaStream_t s, int nslices, int M, int N, int K,
                  size_t work_bytes, cplx* part, size_t part_elems, int* err,
                  SliceBCache* bc, SliceBCache* ac, int64_t upper) {
   if (M <= 0 || N <= 0) return;
-  CVS_REQUIRE(nslices == 4 || nslices == 7, -1, "zgemm_slice: 4 or 7 slices");
+  CVS_REQUIRE(nslices == 4 || nslices == 7 || nslices == 8, -1, "zgemm_slice: 4, 7 or 8 slices");
   CVS_REQUIRE(!ac || nslices == 4, -1, "zgemm_slice: cached A needs 4 slices");
   SDims d = sdims_of(M, N, K, nslices, bc != nullptr, ac != nullptr);
   CVS_REQUIRE(work_bytes >= d.a_bytes + d.b_bytes + d.e_bytes, -1,
@@ -1652,12 +1726,16 @@ void zgemm_slice(cudaStream_t s, int nslices, int M, int N, int K,
                          pair_smem<4>());
     cudaFuncSetAttribute(tc_slice_pair_kernel<7>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          pair_smem<7>());
+    cudaFuncSetAttribute(tc_slice_pair_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         pair_smem<8>());
     cudaFuncSetAttribute(tc_slice4r_kernel,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, R_SMEM);
   });
   auto pack_a = [&](int Kc, int k0, int Kp, int* e, __nv_bfloat16* out) {
     if (nslices == 4)
       pack_lines<4, false>(s, A, M, Kc, k0, d.Mp, Kp, e, d.Mp, out);
+    else if (nslices == 8)
+      pack_lines<8, false>(s, A, M, Kc, k0, d.Mp, Kp, e, d.Mp, out);
     else
       pack_lines<7, false>(s, A, M, Kc, k0, d.Mp, Kp, e, d.Mp, out);
   };
@@ -1665,6 +1743,8 @@ void zgemm_slice(cudaStream_t s, int nslices, int M, int N, int K,
   auto pack_b = [&](int Kc, int k0, int Kp, int* e, __nv_bfloat16* out) {
     if (nslices == 4)
       pack_lines<4, true>(s, trans(B), N, Kc, k0, d.Np2 / 2, Kp, e, eb_n, out);
+    else if (nslices == 8)
+      pack_lines<8, true>(s, trans(B), N, Kc, k0, d.Np2 / 2, Kp, e, eb_n, out);
     else
       pack_lines<7, true>(s, trans(B), N, Kc, k0, d.Np2 / 2, Kp, e, eb_n, out);
   };
@@ -1720,6 +1800,9 @@ void zgemm_slice(cudaStream_t s, int nslices, int M, int N, int K,
     const int tok = kstats_begin(s, K_TC_SLICE, 8.0 * M * N * (double)Kc);
     if (pl.pair && nslices == 4) {
       launch_pair<4>(s, ma, mb, mb2, kpa, ka_off, kpb, kb_off, nkb, zl, nz, M, N, eAc, eBc, alpha,
+                     beta_c, C, pp, upper, err);
+    } else if (nslices == 8) {
+      launch_pair<8>(s, ma, mb, mb2, kpa, ka_off, kpb, kb_off, nkb, zl, nz, M, N, eAc, eBc, alpha,
                      beta_c, C, pp, upper, err);
     } else if (pl.pair) {
       launch_pair<7>(s, ma, mb, mb2, kpa, ka_off, kpb, kb_off, nkb, zl, nz, M, N, eAc, eBc, alpha,

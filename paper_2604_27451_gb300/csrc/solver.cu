@@ -375,6 +375,22 @@ void gemm64(cvsadc_ctx* c, int M, int N, int K, double alpha, View A,
             c->s_kpart.bytes / sizeof(cplx));
 }
 
+// C = A B with 8 slices: FP64 accuracy on the tensor cores
+void gemm_slice8(cvsadc_ctx* c, int M, int N, int K, View A, View B, View C) {
+  A = checked(A);
+  B = checked(B);
+  C = checked(C);
+  check_view(A, M, K, 1, "A");
+  check_view(B, K, N, 1, "B");
+  check_view(C, M, N, 1, "C");
+  const size_t need = slice_workspace_bytes(M, N, K, 8);
+  c->s_tc.ensure(need);
+  zgemm_slice(c->stream, 8, M, N, K, 1.0, A, B, 0.0, C, c->s_tc.p, need, c->s_kpart.c(),
+              c->s_kpart.bytes / sizeof(cplx), c->err_dev);
+}
+// bytes of packed rows of B^P that the rotation into natural spinors holds
+constexpr size_t ROT_PACK = (size_t)512 << 20;
+
 void copyv(cvsadc_ctx* c, int M, int N, double alpha, View src, View dst) {
   src = checked(src);
   dst = checked(dst);
@@ -790,27 +806,58 @@ void build_fns(cvsadc_ctx* c, int prec, double tau) {
   // rotate B^P (and dipoles): occupied rows/cols unchanged, virtual with U
   const int n2 = o + vk;
   const int64_t nn = (int64_t)n * n, nn2 = (int64_t)n2 * n2;
+  // Slice precisions rotate with 8 slices (57 bits below a line's largest
+  // component, exact sums).  Against extended precision their error is 0.8e-16
+  // of the result's norm on 300 x 200 by 200 x 150 with Gaussian entries or a
+  // unitary factor, the FP64 kernels' 4.7e-16; and the FP64 pipes were the
+  // bound of this step: 1000 matrices of 246 x 246, 200 virtuals into 150:
+  // 99 -> 5.6 ms.  Small rotations stay on the FP64 kernels, by the rule of
+  // gemm().
+  const bool slices = prec != CVSADC_FP64 && tc_available() && vk >= 32 && v >= 64;
   auto rotate = [&](const cplx* src, int64_t nmat, DBuf& dst) {
     dst.ensure((size_t)nmat * nn2 * sizeof(cplx));
-    DBuf tmp;
-    tmp.ensure((size_t)nmat * n * vk * sizeof(cplx));
     const cplx* U = c->fns_U.c();
     // oo block copy, rows (P, i) of all matrices at once
     copyv(c, (int)(nmat * o), o, 1.0, rows2(view(src, 0, 1), nn, n, o),
           rows2(view(dst.c(), 0, 1), nn2, n2, o));
-    // tmp[P][p][b'] = sum_b src[P][p][o+b] U[b][b']   (all rows p)
-    gemm(c, CVSADC_FP64, n, vk, v, 1.0,
-         batched(view(src + o, n, 1), nn), view(U, vk, 1), 0.0,
-         batched(view(tmp.p, vk, 1), (int64_t)n * vk), (int)nmat);
-    // ov block: rows i < o of every matrix
-    copyv(c, (int)(nmat * o), vk, 1.0, rows2(view(tmp.c(), 0, 1), (int64_t)n * vk, vk, o),
-          rows2(view(dst.c() + o, 0, 1), nn2, n2, o));
-    // vv block: U^H tmp[P][o:][:], Hermitian: the tiles on and above the
-    // diagonal; then the rest of the rows o .. from their mirror images
-    gemm(c, CVSADC_FP64, vk, vk, v, 1.0,
-         conj_of(trans(view(U, vk, 1))),
-         batched(view(tmp.c() + (int64_t)o * vk, vk, 1), (int64_t)n * vk), 0.0,
-         batched(view(dst.c() + (int64_t)o * n2 + o, n2, 1), nn2), (int)nmat, false, false, 0);
+    const bool tc = slices && (double)nmat * n * vk * v >= 1e7;
+    // nb matrices at a time: as many as keep the packed rows within ROT_PACK
+    // (some 20 rounds of tiles) and in the scratch of the amplitudes' product
+    int64_t nb = nmat;
+    if (tc) {
+      const size_t fixed = slice_workspace_bytes(0, vk, v, 8);
+      const size_t per = slice_workspace_bytes(n, vk, v, 8) - fixed;
+      const size_t have = std::min(ROT_PACK, std::max(c->s_tc.bytes, ROT_PACK / 16)) - fixed;
+      nb = std::max<int64_t>(1, std::min<int64_t>(nmat, (int64_t)(have / per)));
+    }
+    DBuf tmp;
+    tmp.ensure((size_t)nb * n * vk * sizeof(cplx));
+    for (int64_t p0 = 0; p0 < nmat; p0 += nb) {
+      const int64_t np = std::min(nb, nmat - p0);
+      const cplx* sp = src + p0 * nn;
+      cplx* dp = dst.c() + p0 * nn2;
+      // tmp[P][p][b'] = sum_b src[P][p][o+b] U[b][b']   (all rows p)
+      // vv block: sum_a conj(U[a][a']) tmp[P][o+a][b']
+      if (tc) {
+        gemm_slice8(c, (int)(np * n), vk, v, view(sp + o, n, 1), view(U, vk, 1),
+                    view(tmp.p, vk, 1));
+        gemm_slice8(c, (int)(np * vk), vk, v,
+                    rows2(view(tmp.c() + (int64_t)o * vk, 0, vk), (int64_t)n * vk, 1, vk),
+                    conj_of(view(U, vk, 1)),
+                    rows2(view(dp + (int64_t)o * n2 + o, 0, n2), nn2, 1, vk));
+      } else {
+        gemm(c, CVSADC_FP64, n, vk, v, 1.0, batched(view(sp + o, n, 1), nn), view(U, vk, 1), 0.0,
+             batched(view(tmp.p, vk, 1), (int64_t)n * vk), (int)np);
+        // Hermitian: the tiles on and above the diagonal
+        gemm(c, CVSADC_FP64, vk, vk, v, 1.0, conj_of(trans(view(U, vk, 1))),
+             batched(view(tmp.c() + (int64_t)o * vk, vk, 1), (int64_t)n * vk), 0.0,
+             batched(view(dp + (int64_t)o * n2 + o, n2, 1), nn2), (int)np, false, false, 0);
+      }
+      // ov block: rows i < o of every matrix
+      copyv(c, (int)(np * o), vk, 1.0, rows2(view(tmp.c(), 0, 1), (int64_t)n * vk, vk, o),
+            rows2(view(dp + o, 0, 1), nn2, n2, o));
+    }
+    // the rest of the rows o .. from their mirror images
     mirror_fill(c->stream, dst.c(), n2, 0, o, n2, true, nmat, nn2);
   };
   DBuf Bn;

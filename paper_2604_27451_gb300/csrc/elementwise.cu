@@ -191,17 +191,20 @@ __device__ __forceinline__ double reciprocal(double x) {
 // mirror, stages both in shared memory (coalesced rows) and writes
 //   X[al][i][b][j] <- <ab||ij> = (a i|b j) - (a j|b i)
 //   T[al][i][b][j]  = <ab||ij> / (e_i + e_j - e_a - e_b)
-// for both tiles.  part[block] = the block's share of E_MP2 = 1/4 sum |g|^2 /
-// den.
+// for both tiles.  (a i|b j) = (b j|a i), so for b of the band's own square
+// X need only hold b > a: <ba||ij> = -<ab||ij> goes to [bl][i][a][j] (b = a0 +
+// bl) as well, <aa||ij> = 0, and the CTAs of b < a have nothing to do.
+// part[block] = the block's share of E_MP2 = 1/4 sum |g|^2 / den.
 //
 // Bounded by FP64 operations (two per SM and cycle), so everything is done
 // once per unordered pair (i, j): g_ji = -g_ij and t_ji = -t_ij exactly, with
 // one reciprocal for t and the energy (14 operations a pair), and the tile
 // edge divides o evenly so that few lanes idle.  Medium workload (66 occupied,
-// 300 virtuals, 18.8 GB): 8.7 ms, 27 ms with two divisions per element.
+// 300 virtuals, 18.8 GB): 5.7 ms; 8.7 ms, and 3.0 ms to fill in X for b < a,
+// before that square was halved; 27 ms with two divisions per element.
 constexpr int TB2 = 32;
 __global__ void __launch_bounds__(256)
-    t2_band_ip_kernel(cplx* __restrict__ X, cplx* __restrict__ T, int a0, int o, int v,
+    t2_band_ip_kernel(cplx* __restrict__ X, cplx* __restrict__ T, int a0, int nb, int o, int v,
                       const double* __restrict__ eps, int ntile, int te,
                       double* __restrict__ part) {
   __shared__ cplx sa[TB2][TB2 + 1], sb[TB2][TB2 + 1];
@@ -211,6 +214,13 @@ __global__ void __launch_bounds__(256)
   const int64_t ab = blk / npt;
   const int b = (int)(ab % v);
   const int al = (int)(ab / v);
+  // b's place in the band's own square: below the diagonal, on it, above it
+  const int bl = b - a0;
+  if (bl >= 0 && bl < al) {
+    if (threadIdx.x == 0) part[blk] = 0.0;
+    return;
+  }
+  const bool zero = bl == al, mir = bl > al && bl < nb;
   int ti = 0, rem = tp;
   while (rem >= ntile - ti) {
     rem -= ntile - ti;
@@ -223,6 +233,28 @@ __global__ void __launch_bounds__(256)
   const int64_t vo = (int64_t)v * o;
   cplx* Xa = X + (int64_t)al * o * vo + (int64_t)b * o;  // (i, j) -> i vo + j
   cplx* Ta = T + (int64_t)al * o * vo + (int64_t)b * o;
+  // from element (i, j) of [al][.][b][.] to the one of [bl][.][a][.]
+  const int64_t m = ((int64_t)bl * o * vo + (int64_t)(a0 + al) * o) -
+                    ((int64_t)al * o * vo + (int64_t)b * o);
+  auto store = [&](int i, int j, cplx g, cplx t) {
+    const int64_t at = (int64_t)i * vo + j;
+    Xa[at] = g;
+    Ta[at] = t;
+    if (mir) {
+      Xa[at + m] = cmake(-g.x, -g.y);
+      Ta[at + m] = cmake(-t.x, -t.y);
+    }
+  };
+  if (zero) {
+    for (int e = threadIdx.x; e < te * te; e += 256) {
+      const int r = e / te, c = e % te;
+      const cplx z = cmake(0.0, 0.0);
+      if (r < ni && c < nj) store(i0 + r, j0 + c, z, z);
+      if (!dg && r < nj && c < ni) store(j0 + r, i0 + c, z, z);
+    }
+    if (threadIdx.x == 0) part[blk] = 0.0;
+    return;
+  }
   for (int e = threadIdx.x; e < te * te; e += 256) {
     const int r = e / te, c = e % te;
     if (r < ni && c < nj) sa[r][c] = Xa[(int64_t)(i0 + r) * vo + j0 + c];
@@ -245,8 +277,7 @@ __global__ void __launch_bounds__(256)
       if (r >= ni || c >= nj) continue;
       cplx g, t;
       pair(i0 + r, j0 + c, sa[r][c], sb[c][r], g, t);
-      Xa[(int64_t)(i0 + r) * vo + j0 + c] = g;
-      Ta[(int64_t)(i0 + r) * vo + j0 + c] = t;
+      store(i0 + r, j0 + c, g, t);
       sa[r][c] = t;
       sb[c][r] = cmake(-g.x, -g.y);
     }
@@ -255,8 +286,7 @@ __global__ void __launch_bounds__(256)
       const int r = e / te, c = e % te;  // (j0 + r, i0 + c)
       if (r >= nj || c >= ni) continue;
       const cplx t = sa[c][r];
-      Xa[(int64_t)(j0 + r) * vo + i0 + c] = sb[r][c];
-      Ta[(int64_t)(j0 + r) * vo + i0 + c] = cmake(-t.x, -t.y);
+      store(j0 + r, i0 + c, sb[r][c], cmake(-t.x, -t.y));
     }
   } else {
     // the pairs r < c, counted row by row
@@ -280,12 +310,11 @@ __global__ void __launch_bounds__(256)
     for (int e = threadIdx.x; e < te * te; e += 256) {
       const int r = e / te, c = e % te;
       if (r >= ni || c >= ni) continue;
-      Xa[(int64_t)(i0 + r) * vo + i0 + c] = sa[r][c];
-      Ta[(int64_t)(i0 + r) * vo + i0 + c] = sb[r][c];
+      store(i0 + r, i0 + c, sa[r][c], sb[r][c]);
     }
   }
   const double sum = block_sum(acc);
-  if (threadIdx.x == 0) part[blk] = 0.5 * sum;
+  if (threadIdx.x == 0) part[blk] = (mir ? 1.0 : 0.5) * sum;
 }
 
 // X[m][off + q] = X[q][off + m] (conjugated if CONJ) for m0 <= m < m1, q < m:
@@ -321,11 +350,16 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// *out += sum of in[0..n)
-__global__ void reduce_sum_add_kernel(const double* in, int64_t n, double* out) {
-  double acc = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) acc += in[i];
-  double s = block_sum(acc);
+// *out += sum of in[0..n), one block: four loads in flight per thread (540000
+// partials of the medium workload: 161 us, 350 us with one and 256 threads)
+__global__ void __launch_bounds__(1024) reduce_sum_add_kernel(const double* in, int64_t n,
+                                                              double* out) {
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int64_t i = threadIdx.x; i < n; i += 4096)
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i + q * 1024 < n) acc[q] += in[i + q * 1024];
+  double s = block_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
   if (threadIdx.x == 0) *out += s;
 }
 
@@ -1106,10 +1140,10 @@ void t2_band_inplace(cudaStream_t s, cplx* X, cplx* T, int a0, int nb, int o,
   const int nt = (o + TB2 - 1) / TB2;
   const int64_t nblk = t2_band_ip_blocks(nb, o, v);
   CVS_REQUIRE(nblk < (1LL << 31), -1, "t2_band_inplace: band too large");
-  t2_band_ip_kernel<<<(unsigned)nblk, 256, 0, s>>>(X, T, a0, o, v, eps, nt, (o + nt - 1) / nt,
+  t2_band_ip_kernel<<<(unsigned)nblk, 256, 0, s>>>(X, T, a0, nb, o, v, eps, nt, (o + nt - 1) / nt,
                                                    part);
   CVS_CHECK_LAUNCH();
-  reduce_sum_add_kernel<<<1, 256, 0, s>>>(part, nblk, emp2);
+  reduce_sum_add_kernel<<<1, 1024, 0, s>>>(part, nblk, emp2);
   CVS_CHECK_LAUNCH();
 }
 

@@ -85,7 +85,8 @@ void t2_band(cudaStream_t s, const cplx* V, int a0, int na, int o, int v,
              const double* eps, cplx* t2, cplx* g2, double* part, int nblk);
 // Band transform in place: X [al][i][b][j] = (a i|b j) for a = a0 + al
 // becomes <ab||ij>, T (same layout) = t^{ab}_{ij}; *emp2 (device) += the
-// band's share of E_MP2.  part must hold t2_band_ip_blocks(nb, o, v)
+// band's share of E_MP2.  Of the square of the band's own b, a0 <= b < a0 +
+// nb, X need only hold b > a.  part must hold t2_band_ip_blocks(nb, o, v)
 // doubles.
 int64_t t2_band_ip_blocks(int nb, int o, int v);
 void t2_band_inplace(cudaStream_t s, cplx* X, cplx* T, int a0, int nb, int o,

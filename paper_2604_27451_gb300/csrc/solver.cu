@@ -526,10 +526,9 @@ double t2_bands(cvsadc_ctx* c, int prec, const cplx* B, const double* eps, int o
     const int nb = std::min(na, v - a0);
     View A = rows2(view(B + (int64_t)(o + a0) * n, 0, nn), n, 1, o);
     View Bv = cols2(view(B + (int64_t)o * n, nn, 0), n, 1, o);
-    // (ai|bj) = (bj|ai): the square of the band's own b is symmetric
+    // (ai|bj) = (bj|ai): of the square of the band's own b, b > a will do
     gemm(c, prec, nb * o, (int)vo, L, 1.0, A, Bv, 0.0, view(X.p, vo, 1), 1, false, false,
          (int64_t)a0 * o);
-    mirror_fill(c->stream, X.c(), vo, (int64_t)a0 * o, 0, nb * o, false);
     t2_band_inplace(c->stream, X.c(), T.c(), a0, nb, o, v, eps, part.d(), dE);
     use(Band{a0, nb, T.c(), X.c()});
   }

@@ -87,6 +87,9 @@ struct View {
   int64_t batch;  // batch stride
   int32_t conj;
   int64_t ext;  // elements addressable from p (-1: not checked)
+  // offsets of the c_lo inner columns (each below cs_hi) in place of multiples
+  // of cs_lo; read by the packing of the slice products only
+  const int* ctab = nullptr;
 };
 
 static inline View view(const void* p, int64_t rs, int64_t cs,

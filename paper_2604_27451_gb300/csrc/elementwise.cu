@@ -350,6 +350,14 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// offsets k stride + l of the pairs k < l < o, row by row
+__global__ void pair_offsets_kernel(int o, int stride, int* out) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < o * o; e += gridDim.x * blockDim.x) {
+    const int k = e / o, l = e % o;
+    if (k < l) out[k * (2 * o - k - 1) / 2 + l - k - 1] = k * stride + l;
+  }
+}
+
 // *out += sum of in[0..n), one block: four loads in flight per thread (540000
 // partials of the medium workload: 161 us, 350 us with one and 256 threads)
 __global__ void __launch_bounds__(1024) reduce_sum_add_kernel(const double* in, int64_t n,
@@ -1106,6 +1114,11 @@ void hermiticity_quick(cudaStream_t s, const cplx* B, int n, int64_t nmat, doubl
   const int64_t nblk = nmat * (nt * (nt + 1) / 2);
   CVS_REQUIRE(nblk < (1LL << 31), -1, "hermiticity_quick: too many tiles");
   herm_quick_kernel<<<(unsigned)nblk, 256, 0, s>>>(B, n, nt, (unsigned long long*)out_dev);
+  CVS_CHECK_LAUNCH();
+}
+
+void pair_offsets(cudaStream_t s, int o, int stride, int* out) {
+  pair_offsets_kernel<<<grid1d((int64_t)o * o, 256), 256, 0, s>>>(o, stride, out);
   CVS_CHECK_LAUNCH();
 }
 

@@ -1145,8 +1145,8 @@ __device__ __forceinline__ int exp_field(double x) {
 // column offset of a view for an int column index (32-bit index math)
 __device__ __forceinline__ int64_t vcol32(const View& v, int c) {
   if (v.c_lo == INT32_MAX) return (int64_t)c * v.cs_lo;
-  const int h = c / v.c_lo;
-  return (int64_t)h * v.cs_hi + (int64_t)(c - h * v.c_lo) * v.cs_lo;
+  const int h = c / v.c_lo, r = c - h * v.c_lo;
+  return (int64_t)h * v.cs_hi + (v.ctab ? (int64_t)v.ctab[r] : (int64_t)r * v.cs_lo);
 }
 
 // Operands are packed line by line: rows of A, columns of B (a transposed

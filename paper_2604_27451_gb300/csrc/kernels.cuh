@@ -83,6 +83,8 @@ void hermiticity_quick(cudaStream_t s, const cplx* B, int n, int64_t nmat, doubl
 // 1/4 |g2|^2 / den into per-block partials part[nblk].
 void t2_band(cudaStream_t s, const cplx* V, int a0, int na, int o, int v,
              const double* eps, cplx* t2, cplx* g2, double* part, int nblk);
+// out[p] = k stride + l of the o (o - 1) / 2 pairs k < l < o
+void pair_offsets(cudaStream_t s, int o, int stride, int* out);
 // Band transform in place: X [al][i][b][j] = (a i|b j) for a = a0 + al
 // becomes <ab||ij>, T (same layout) = t^{ab}_{ij}; *emp2 (device) += the
 // band's share of E_MP2.  Of the square of the band's own b, a0 <= b < a0 +

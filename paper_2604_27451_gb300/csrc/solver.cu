@@ -359,6 +359,7 @@ void gemm(cvsadc_ctx* c, int prec, int M, int N, int K, double alpha, View A,
     }
     return;
   }
+  CVS_REQUIRE(!A.ctab && !B.ctab, -1, "gemm: a column table needs a slice product");
   zgemm_f64(c->stream, M, N, K, alpha, A, B, beta, C, batch, c->s_kpart.c(),
             c->s_kpart.bytes / sizeof(cplx), upper);
 }
@@ -577,11 +578,32 @@ void build_m11(cvsadc_ctx* c, int prec) {
       copyv(c, nc, v, 1.0, view(c->dip.c() + (int64_t)x * nn + (int64_t)o * n, 1, n),
             view(c->F.c() + (int64_t)x * N, v, 1));
   }
+  // offsets of the pairs k < l in a band's [.][k][.][l]
+  constexpr int64_t FOLD_MIN = 1 << 18;
+  const int pairs = o * (o - 1) / 2;
+  const bool fold = (prec == CVSADC_MIXED_SLICE4 || prec == CVSADC_FP64_SLICE7) &&
+                    tc_available() && v > 64 && (int64_t)v * o * o >= FOLD_MIN &&
+                    ovo <= INT32_MAX;
+  DBuf poff;
+  if (fold) {
+    poff.ensure((size_t)pairs * sizeof(int));
+    pair_offsets(c->stream, o, (int)vo, (int*)poff.p);
+  }
   c->emp2 = t2_bands(c, prec, B, c->eps.d(), o, v, L, [&](const Band& b) {
     const double beta = b.a0 == 0 ? 0.0 : 1.0;
-    // X_ab += sum_{(c,k),l} t^{ca}_{kl} conj(<cb||kl>)   (the Ivv piece)
-    gemm(c, prec, v, v, b.nb * o * o, 1.0, cols2(view(b.T, o, 0), vo, 1, o),
-         conj_of(rows2(view(b.G, 0, o), vo, 1, o)), beta, view(X, v, 1));
+    // X_ab += sum_{c,k,l} t^{ca}_{kl} conj(<cb||kl>)   (the Ivv piece); both
+    // change sign with k and l exchanged, so the slice products take k < l
+    // twice where the sum is long enough to matter (300 virtuals, 66 occupied:
+    // 10.7 ms with the packing, 21.5 ms over all k, l; below 2^18 terms the
+    // whole piece is well under a millisecond)
+    if (fold && (int64_t)b.nb * o * o >= FOLD_MIN) {
+      View t = cols2(view(b.T, o, 0), ovo, 1, pairs), g = cols2(view(b.G, o, 0), ovo, 1, pairs);
+      t.ctab = g.ctab = (const int*)poff.p;
+      gemm(c, prec, v, v, b.nb * pairs, 2.0, t, conj_of(trans(g)), beta, view(X, v, 1));
+    } else {
+      gemm(c, prec, v, v, b.nb * o * o, 1.0, cols2(view(b.T, o, 0), vo, 1, o),
+           conj_of(rows2(view(b.G, 0, o), vo, 1, o)), beta, view(X, v, 1));
+    }
     // Y_IJ += sum_{c,(d,k)} t^{cd}_{Ik} conj(<cd||Jk>)   (the Joo piece)
     gemm(c, prec, nc, nc, b.nb * (int)vo, 1.0, cols2(view(b.T, vo, 0), ovo, 1, (int)vo),
          conj_of(rows2(view(b.G, 0, vo), ovo, 1, (int)vo)), beta, view(Y, nc, 1));

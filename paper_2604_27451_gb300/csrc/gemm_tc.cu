@@ -1160,7 +1160,8 @@ __device__ __forceinline__ int64_t vcol32(const View& v, int c) {
 // Otherwise (the lines are the contiguous mode: columns of a row-major B,
 // (a, b) rows of B^P) lanes take adjacent lines and walk a segment, so that
 // the warp reads 512 contiguous bytes a step instead of half a sector each.
-constexpr int EXP_SEG = 4096, EXP_SEG_LINES = 64;
+// (942 lines of 5181: 56 us in segments of 4096, 16 us of 1024.)
+constexpr int EXP_SEG = 1024, EXP_SEG_LINES = 64;
 template <bool KFAST>
 __global__ void __launch_bounds__(256) line_exp_kernel(View X, int L, int K, int k0, int* e) {
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -1632,7 +1633,8 @@ SDims sdims_of(int M, int N, int K, int nslices, bool b_cached, bool a_cached = 
 // SLICE4's 128 x 64 tiles: 1.3 us per unit, a CTA per tile, 8 units of start
 // and end: they keep narrow (2 N <= 64) and small products.  K slices need
 // an output that fits the scratch, and cost its way through memory (32 bytes
-// per partial at 6 TB/s) and a launch.
+// per partial at 6 TB/s) and a launch.  Up to 64 of them: 300 x 24 outputs
+// with K = 450000 are 3 tiles (1410 -> 910 us against at most 32).
 struct SlicePlan {
   bool pair;
   int splits;
@@ -1641,7 +1643,7 @@ SlicePlan plan_slices(int nslices, int M, int N, int nkb, size_t part_elems) {
   SlicePlan best{true, 1};
   double tbest = 1e300;
   auto consider = [&](bool pair, double tiles, double workers, double unit, double fixed) {
-    for (int sp = 1; sp <= 32; ++sp) {
+    for (int sp = 1; sp <= 64; ++sp) {
       if (sp > 1 && (nkb / sp < 4 || (size_t)sp * M * N > part_elems)) break;
       const double units = 2.0 * ((nkb + sp - 1) / sp);
       double t = std::ceil(tiles * sp / workers) * (units + fixed) * unit;

@@ -177,8 +177,12 @@ __global__ void t2_band_kernel(const cplx* __restrict__ V, int a0, int na,
 }
 
 // 1 / x to an ulp or so: the hardware's approximation and two Newton steps,
-// half the FP64 operations of a division
+// half the FP64 operations of a division.  Zero, infinite and not-a-number x
+// and those at the ends of the exponent range, where a step would make a NaN
+// of an infinity, divide (told by the exponent bits, on the integer pipe).
 __device__ __forceinline__ double reciprocal(double x) {
+  const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7FFu;
+  if (e - 2u > 2042u) return 1.0 / x;
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
   r = fma(r, fma(-x, r, 1.0), r);

@@ -855,6 +855,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(pair_threads<NS>(), 
         }
       }
     }
+    // The issuers' commits arrive in both CTAs' shared memory on their own
+    // time, the last ones on barriers that no later copy waits for.  Each
+    // producer waits for the last use of every slot, so that its CTA is still
+    // there when they arrive: cluster_sync() does not order them.
+    for (int j = max(0, u - BS); j < u && !fail; ++j)
+      if (!mbar_wait(&emptyB[j % BS], (j / BS) & 1)) fail = 6;
+    for (int j = max(0, ia - AS); j < ia && !fail; ++j)
+      if (!mbar_wait(&emptyA[j % AS], (j / AS) & 1)) fail = 6;
   } else if (warp >= 1 && warp <= NI) {
     if (rank == 0 && lane == 0) {
       const uint32_t dhi = (uint32_t)(sdesc(0) >> 32);

@@ -292,29 +292,6 @@ View rows_from(View v, int64_t m0) {
   return v;
 }
 
-// Whether an M x N output of a long K, of FP64 accuracy in every precision, is
-// cheaper as an 8-slice product.  Modelled times in us: 8 M N K operations at
-// the FP64 kernels' 1.2 TFLOP/s, against packing (rows padded to 128 and
-// columns to 64, 32 and 64 bytes written per k, operands read twice, at 4.5
-// TB/s), the units of plan_slices and a few launches; one vector's blocks and
-// the core x core ones stay FP64.  Whole calls, FP64 kernels against slices,
-// and the errors against quadruple precision (Gaussian entries that decay as
-// exp(-P / 60)):
-//   100 x 24 x 50000     952 ->  297 us   4.4e-16  4.1e-16
-//   157 x 12 x 123245   1667 ->  838 us   4.7e-16  4.3e-16
-//   157 x 18 x 123245   2474 ->  837 us   3.0e-16  2.3e-16
-//    64 x 48 x 22000     528 ->  219 us   3.8e-16  2.8e-16
-// Above 2^17 terms the digits cut off below a line's largest element add up
-// (200 x 12 x 200000: 2.9e-16 FP64, 3.5e-16 slices), so those stay FP64.
-bool slice8_pays(int M, int N, int K) {
-  if (K > 1 << 17) return false;
-  const double mp = (M + 127) / 128 * 128, np = (N + 63) / 64 * 64;
-  const double tiles = std::ceil(M / 256.0) * std::ceil(2 * N / 64.0);
-  const double pack = K * (32.0 * mp + 64.0 * np + 32.0 * (M + N)) / 4.5e6;
-  const double mma = (K / 32.0 / std::min(64.0, 76.0 / tiles) + 7.0) * 3.75;
-  return 25.0 + pack + mma < 0.8 * (8.0 * M * N * (double)K / 1.2e6);
-}
-
 // cache_b / cache_a: B / A is the same view of B^P on every call (the sigma
 // products), so its packed slices may be kept.  upper: as in zgemm_f64
 void gemm(cvsadc_ctx* c, int prec, int M, int N, int K, double alpha, View A,
@@ -328,16 +305,10 @@ void gemm(cvsadc_ctx* c, int prec, int M, int N, int K, double alpha, View A,
   check_view(C, M, N, batch, "C");
   // the tensor-core path pays a packing pass per operand: keep it for
   // contractions with enough work per packed element
-  // small outputs with a long K: FP64 accuracy, on whichever pipe is faster
+  // small outputs with a long K: FP64 in every precision (slices would cut
+  // what is small beside the largest element of its row or column, and read
+  // infinities and not-a-numbers as digits)
   const bool small = (int64_t)M * N <= 4096 && M + N <= 384 && K >= 4096;
-  if (small && batch == 1 && upper < 0 && tc_available() &&
-      (prec == CVSADC_MIXED_SLICE4 || prec == CVSADC_FP64_SLICE7) && slice8_pays(M, N, K)) {
-    const size_t need = slice_workspace_bytes(M, N, K, 8);
-    c->s_tc.ensure(need);
-    zgemm_slice(c->stream, 8, M, N, K, alpha, A, B, beta, C, c->s_tc.p, need, c->s_kpart.c(),
-                c->s_kpart.bytes / sizeof(cplx), c->err_dev);
-    return;
-  }
   const bool tc = !small && prec != CVSADC_FP64 && M >= 32 && K >= 64 &&
                   (double)M * N * K >= 1e7;
   if (tc) {
@@ -2913,11 +2884,6 @@ double estimate_bytes(const cvsadc_params* p) {
                      ws(g * N1, L, wv, ns), ws(g * wv, L, N1, ns), ws(g * N1, wv, L, ns),
                      ws(N1, g * wv, L, ns)})
       w = std::max(w, s);
-    // v x (core, vector) outputs summed over (P, a): 8 slices (slice8_pays)
-    const double nmax = std::min(4096.0 / v, 384.0 - v);
-    if (ns && p->precision != CVSADC_FP64 && nmax >= 1 && L * v <= 2e9 &&
-        slice8_pays((int)v, (int)nmax, (int)(L * v)))
-      w = std::max(w, ws(v, nmax, L * v, 8));
     // the preconditioner's contractions run as 4-slice products
     if (schur_on) {
       const double v3 = v * v * v;

@@ -239,12 +239,12 @@ __global__ void __launch_bounds__(NT)
 typedef void (*F64Kernel)(int, int, int, double, View, View, double, View, int, int, int, int,
                           int, int64_t, cplx*);
 struct F64Shape {
-  int tm, tn, bk;
+  int tm, tn, bk, kx;
   double eff;
   F64Kernel fn;
 };
 #define CVS_F64(TY, TX, RM, RN, BK, ST, EFF) \
-  {TY * RM, TX * RN, BK, EFF, zgemm_f64_kernel<TY, TX, RM, RN, BK, ST>}
+  {TY * RM, TX * RN, BK, NT / (TY * TX), EFF, zgemm_f64_kernel<TY, TX, RM, RN, BK, ST>}
 // with the share of the FP64 rate each holds on 1000 products of 246 x 165 x
 // 200 (its padding and whole k steps counted as work)
 const F64Shape F64_SHAPES[] = {
@@ -322,10 +322,36 @@ __global__ void splitk_reduce_kernel(int M, int N, int nz, const cplx* part,
   for (int64_t idx = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / W; idx < MN;
        idx += (int64_t)gridDim.x * blockDim.x / W) {
     double sr = 0, si = 0;
-    for (int z = lane; z < nz; z += W) {
-      cplx v = part[z * MN + idx];
-      sr += v.x;
-      si += v.y;
+    if (nz <= 4 * W) {
+      for (int z = lane; z < nz; z += W) {
+        const cplx v = part[z * MN + idx];
+        sr += v.x;
+        si += v.y;
+      }
+    } else {
+      // eight running sums, added pairwise (1217 x 4 x 901, 29 slices: rms error
+      // 3.3e-16 -> 2.9e-16; their additions cost 30 us a single-vector sigma
+      // of 6/33/157/785 where there are only a few slices)
+      double r8[8], i8[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) r8[q] = i8[q] = 0.0;
+      for (int z0 = lane; z0 < nz; z0 += 8 * W)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          if (z0 + q * W >= nz) break;
+          const cplx v = part[(z0 + q * W) * MN + idx];
+          r8[q] += v.x;
+          i8[q] += v.y;
+        }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < o; ++q) {
+          r8[q] += r8[q + o];
+          i8[q] += i8[q + o];
+        }
+      sr = r8[0];
+      si = i8[0];
     }
 #pragma unroll
     for (int o = W / 2; o > 0; o >>= 1) {
@@ -371,10 +397,16 @@ void zgemm_f64(cudaStream_t s, int M, int N, int K, double alpha, View A,
   const int bk = p.shape->bk;
   const int kchunk = ((K + p.splits - 1) / p.splits + bk - 1) / bk * bk;
   const int nz = (K + kchunk - 1) / kchunk;
-  // long contractions in chains of 128 (45 x 60 x 5000: 6.1e-16 of the result
-  // in chains of 625, 3.1e-16 in these); short ones as they come (two more
-  // additions per output cost up to 8 % of the small tiles at K = 200)
-  const int period = K >= 4096 ? 128 / bk : INT32_MAX;
+  // Long contractions in chains of 32 terms a thread, short ones of a few
+  // columns in chains of 16 (kx groups of threads take every kx-th k); others
+  // as they come (two more additions per output cost up to 8 % of the small
+  // tiles at K = 200).  Rms error against double-double sums of Gaussian
+  // entries, in these chains and in chains of 128 or whole K slices:
+  //   64 x 48 x 22000   3.1e-16 (4.0e-16)   1800 x 4 x 1800   2.5e-16 (7.2e-16)
+  //   157 x 6 x 123245  3.4e-16 (4.5e-16)   1217 x 4 x 901    2.2e-16 (3.3e-16)
+  // The third takes 849 us, 844 us in chains of 128 and 863 us of 16.
+  const int chain = K >= 4096 ? 32 : 16;
+  const int period = K >= 4096 || N <= 8 ? std::max(1, chain * p.shape->kx / bk) : INT32_MAX;
   const int ntn = (N + p.shape->tn - 1) / p.shape->tn;
   const int64_t tiles = (int64_t)ntn * ((M + p.shape->tm - 1) / p.shape->tm);
   CVS_REQUIRE(tiles <= INT32_MAX, -1, "zgemm_f64: output too large");

@@ -176,19 +176,6 @@ __global__ void t2_band_kernel(const cplx* __restrict__ V, int a0, int na,
   if (threadIdx.x == 0) part[blockIdx.x] += s;
 }
 
-// 1 / x to an ulp or so: the hardware's approximation and two Newton steps,
-// half the FP64 operations of a division.  Zero, infinite and not-a-number x
-// and those at the ends of the exponent range, where a step would make a NaN
-// of an infinity, divide (told by the exponent bits, on the integer pipe).
-__device__ __forceinline__ double reciprocal(double x) {
-  const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7FFu;
-  if (e - 2u > 2042u) return 1.0 / x;
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
-}
-
 // In-place band transform.  X holds a band [al][i][b][j] = (a i | b j)
 // (a = a0 + al, i, j occupied, b virtual).  Each CTA takes one (al, b) and
 // one pair of te x te tiles (i-tile ti <= j-tile tj) together with its
@@ -202,10 +189,10 @@ __device__ __forceinline__ double reciprocal(double x) {
 //
 // Bounded by FP64 operations (two per SM and cycle), so everything is done
 // once per unordered pair (i, j): g_ji = -g_ij and t_ji = -t_ij exactly, with
-// one reciprocal for t and the energy (14 operations a pair), and the tile
-// edge divides o evenly so that few lanes idle.  Medium workload (66 occupied,
-// 300 virtuals, 18.8 GB): 5.7 ms; 8.7 ms, and 3.0 ms to fill in X for b < a,
-// before that square was halved; 27 ms with two divisions per element.
+// one division for t and the energy, and the tile edge divides o evenly so
+// that few lanes idle.  Medium workload (66 occupied, 300 virtuals; 3.1 GB
+// read and 12.5 GB written): 5.9 ms; 8.7 ms, and 3.0 ms to fill in X for
+// b < a, before that square was halved; 27 ms with two divisions per element.
 constexpr int TB2 = 32;
 __global__ void __launch_bounds__(256)
     t2_band_ip_kernel(cplx* __restrict__ X, cplx* __restrict__ T, int a0, int nb, int o, int v,
@@ -271,7 +258,7 @@ __global__ void __launch_bounds__(256)
   // t replaces whichever the second pass can do without
   auto pair = [&](int i, int j, cplx xij, cplx xji, cplx& g, cplx& t) {
     g = csub(xij, xji);
-    const double inv = reciprocal(eps[i] + eps[j] - eab);
+    const double inv = 1.0 / (eps[i] + eps[j] - eab);
     t = cscale(g, inv);
     acc = fma(fma(g.x, g.x, g.y * g.y), inv, acc);
   };

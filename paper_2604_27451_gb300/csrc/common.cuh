@@ -87,9 +87,12 @@ struct View {
   int64_t batch;  // batch stride
   int32_t conj;
   int64_t ext;  // elements addressable from p (-1: not checked)
-  // offsets of the c_lo inner columns (each below cs_hi) in place of multiples
-  // of cs_lo; read by the packing of the slice products only
+  // offsets of the r_lo inner rows / c_lo inner columns in place of multiples
+  // of rs_lo / cs_lo, and the largest of them; columns' tables are read by the
+  // packing of the slice products only
+  const int* rtab = nullptr;
   const int* ctab = nullptr;
+  int64_t rtab_max = 0, ctab_max = 0;
 };
 
 static inline View view(const void* p, int64_t rs, int64_t cs,
@@ -119,6 +122,17 @@ static inline View cols2(View v, int64_t hi, int64_t lo, int32_t lo_extent) {
   v.c_lo = lo_extent;
   return v;
 }
+// cols2 with the inner offsets read from a device table of lo_extent
+// entries in [0, tab_max]
+static inline View cols_table(View v, int64_t hi, const int* tab, int64_t tab_max,
+                              int32_t lo_extent) {
+  v.cs_hi = hi;
+  v.cs_lo = 1;
+  v.c_lo = lo_extent;
+  v.ctab = tab;
+  v.ctab_max = tab_max;
+  return v;
+}
 static inline View conj_of(View v) {
   v.conj ^= 1;
   return v;
@@ -134,13 +148,15 @@ static inline View extent(View v, int64_t ext) {
 // Largest element offset a view reaches over rows x cols (x batch).
 static inline int64_t view_max_offset(const View& v, int64_t rows,
                                       int64_t cols, int64_t batch) {
-  auto span = [](int64_t cnt, int64_t hi, int64_t lo, int32_t lo_ext) {
+  auto span = [](int64_t cnt, int64_t hi, int64_t lo, int32_t lo_ext, const int* tab,
+                 int64_t tab_max) {
     if (cnt <= 0) return (int64_t)0;
+    if (tab) return ((cnt - 1) / lo_ext) * hi + tab_max;
     if (lo_ext == INT32_MAX || cnt <= lo_ext) return (cnt - 1) * lo;
     return ((cnt - 1) / lo_ext) * hi + (int64_t)(lo_ext - 1) * lo;
   };
-  return span(rows, v.rs_hi, v.rs_lo, v.r_lo) +
-         span(cols, v.cs_hi, v.cs_lo, v.c_lo) + (batch - 1) * v.batch;
+  return span(rows, v.rs_hi, v.rs_lo, v.r_lo, v.rtab, v.rtab_max) +
+         span(cols, v.cs_hi, v.cs_lo, v.c_lo, v.ctab, v.ctab_max) + (batch - 1) * v.batch;
 }
 // Throws unless every element a rows x cols (x batch) access touches lies
 // inside the view's declared extent.
@@ -167,6 +183,10 @@ static inline View trans(View v) {
   t.cs_hi = v.rs_hi;
   t.cs_lo = v.rs_lo;
   t.c_lo = v.r_lo;
+  t.rtab = v.ctab;
+  t.rtab_max = v.ctab_max;
+  t.ctab = v.rtab;
+  t.ctab_max = v.rtab_max;
   return t;
 }
 

@@ -303,6 +303,8 @@ void gemm(cvsadc_ctx* c, int prec, int M, int N, int K, double alpha, View A,
   check_view(A, M, K, batch, "A");
   check_view(B, K, N, batch, "B");
   check_view(C, M, N, batch, "C");
+  // only the packing of the slice products reads tables, along K
+  CVS_REQUIRE(!A.rtab && !B.ctab && !C.rtab && !C.ctab, -1, "gemm: a table outside K");
   // the tensor-core path pays a packing pass per operand: keep it for
   // contractions with enough work per packed element
   // small outputs with a long K: FP64 in every precision (slices would cut
@@ -311,10 +313,11 @@ void gemm(cvsadc_ctx* c, int prec, int M, int N, int K, double alpha, View A,
   const bool small = (int64_t)M * N <= 4096 && M + N <= 384 && K >= 4096;
   const bool tc = !small && prec != CVSADC_FP64 && M >= 32 && K >= 64 &&
                   (double)M * N * K >= 1e7;
+  const int ns = !tc ? 0 : prec == CVSADC_MIXED_SLICE4 ? 4 : prec == CVSADC_FP64_SLICE7 ? 7 : 0;
+  CVS_REQUIRE(ns || (!A.ctab && !B.rtab), -1, "gemm: a table needs a slice product");
   if (tc) {
     CVS_REQUIRE(tc_available(), CVSADC_EINVAL,
                 "tensor-core precisions need an sm_103 GPU with tcgen05");
-    const int ns = prec == CVSADC_MIXED_SLICE4 ? 4 : prec == CVSADC_FP64_SLICE7 ? 7 : 0;
     SliceBCache* bc = (ns && batch == 1 && cache_b) ? op_cache(c, 0, ns, N, K, B) : nullptr;
     SliceBCache* ac =
         (ns == 4 && batch == 1 && cache_a) ? op_cache(c, 1, ns, M, K, A) : nullptr;
@@ -361,7 +364,6 @@ void gemm(cvsadc_ctx* c, int prec, int M, int N, int K, double alpha, View A,
     }
     return;
   }
-  CVS_REQUIRE(!A.ctab && !B.ctab, -1, "gemm: a column table needs a slice product");
   zgemm_f64(c->stream, M, N, K, alpha, A, B, beta, C, batch, c->s_kpart.c(),
             c->s_kpart.bytes / sizeof(cplx), upper);
 }
@@ -599,8 +601,10 @@ void build_m11(cvsadc_ctx* c, int prec) {
     // 10.7 ms with the packing, 21.5 ms over all k, l; below 2^18 terms the
     // whole piece is well under a millisecond)
     if (fold && (int64_t)b.nb * o * o >= FOLD_MIN) {
-      View t = cols2(view(b.T, o, 0), ovo, 1, pairs), g = cols2(view(b.G, o, 0), ovo, 1, pairs);
-      t.ctab = g.ctab = (const int*)poff.p;
+      const int* tab = (const int*)poff.p;
+      const int64_t last = (int64_t)(o - 2) * vo + o - 1;  // the pair (o - 2, o - 1)
+      const View t = cols_table(view(b.T, o, 0), ovo, tab, last, pairs);
+      const View g = cols_table(view(b.G, o, 0), ovo, tab, last, pairs);
       gemm(c, prec, v, v, b.nb * pairs, 2.0, t, conj_of(trans(g)), beta, view(X, v, 1));
     } else {
       gemm(c, prec, v, v, b.nb * o * o, 1.0, cols2(view(b.T, o, 0), vo, 1, o),

@@ -2905,15 +2905,22 @@ double estimate_bytes(const cvsadc_params* p) {
     b += w;
   }
   b += (double)(8 << 20) * z + 1024;        // split-K scratch
-  // cached slice packs of B^P views (at most min(35 % of free, 64 GB)): the
-  // B operands of the sigma's S and G products, the A operands of its
-  // sigma1^T and Y^T products, and the preconditioner's (aj|bc) product
+  // cached slice packs of B^P views (at most min(35 % of free, 64 GB)), every
+  // slice packed once: lines (a row of A is one, a column of B two) of 2 ns
+  // segments of K bf16 values, padded to the tiles
   {
-    const double pairs = (p->precision == CVSADC_FP64_SLICE7 || needs_refine(p->precision))
-                             ? 10.0 + 28.0 : 10.0;
-    double cb = schur_on ? 8.0 * 10.0 * v * v * L : 0.0;
-    if (p->precision != CVSADC_FP64) cb += 2.0 * 8.0 * pairs * v * v * L;
-    if (p->precision != CVSADC_FP64) cb += 32.0 * v * v * L;
+    auto pack = [](double lines, double pad, double K, int ns) {
+      return std::ceil(lines / pad) * pad * std::ceil(K / 64) * 64 * 4.0 * ns;
+    };
+    double cb = 0.0;
+    // the sigma's B operands (S and G products) and, in 4 slices, its A
+    // operands (sigma1^T and Y^T); the preconditioner's couplings are 4-slice
+    // products in every precision, and mixed ones are refined with 7 slices
+    if (schur_on || p->precision == CVSADC_MIXED_SLICE4)
+      cb += pack(2 * L, 64, wv, 4) + pack(2 * wv, 64, L, 4) + pack(v, 128, v * L, 4) +
+            pack(v * L, 128, v, 4);
+    if (p->precision == CVSADC_FP64_SLICE7 || needs_refine(p->precision))
+      cb += pack(2 * L, 128, wv, 7) + pack(2 * wv, 128, L, 7);
     b += std::min(64e9, cb);
   }
   // Schur-complement preconditioner (when the singles space allows it)

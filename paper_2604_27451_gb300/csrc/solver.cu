@@ -3064,15 +3064,15 @@ int cvsadc_create(cvsadc_ctx** ctx, int device, void* cuda_stream) {
   int rc = guarded(c, [&] {
     init_kernel_attributes();
     c->s_kpart.ensure((size_t)8 << 20 << 4);  // 8 Mi complex = 128 MB
+    CVS_CUDA(cudaHostAlloc((void**)&c->err, 64, cudaHostAllocMapped | cudaHostAllocPortable));
+    *(volatile int*)c->err = 0;
+    CVS_CUDA(cudaHostGetDevicePointer((void**)&c->err_dev, c->err, 0));
     if (cuda_stream) {
       c->stream = (cudaStream_t)cuda_stream;
     } else {
       CVS_CUDA(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
       c->own_stream = true;
     }
-    CVS_CUDA(cudaHostAlloc((void**)&c->err, 64, cudaHostAllocMapped | cudaHostAllocPortable));
-    *(volatile int*)c->err = 0;
-    CVS_CUDA(cudaHostGetDevicePointer((void**)&c->err_dev, c->err, 0));
   });
   if (rc != CVSADC_OK) {
     delete c;

@@ -329,7 +329,8 @@ def run_ours(args):
     if cnt.value > 0 and prec in PRODUCTS:
         achieved = kfl.value / (kms.value / 1e3) / 1e12
         peak = peaks["bf16_tflops"] / PRODUCTS[prec]
-        kname = {"slice4": "tc_slice_pair_kernel", "fp64_slice7": "tc_slice_pair_kernel",
+        kname = {"slice4": "tc_slice_pair_kernel+tc_slice4r_kernel",
+                 "fp64_slice7": "tc_slice_pair_kernel",
                  "bf16x3": "tc_gemm_kernel"}[prec]
         roofline = {"bound": "tensor", "achieved": round(achieved, 2), "peak": round(peak, 2),
                     "unit": "TFLOP/s", "frac": round(achieved / peak, 4),

@@ -76,7 +76,7 @@ extern "C" {
 #define CVSADC_MIXED_SLICE4 2  /* tensor-core GEMMs on exact integer slices:
                                   per-row/column power-of-two scales, four
                                   7-bit slices per value (10 slice products),
-                                  exact FP32 runs of <= 1024 products drained
+                                  exact FP32 runs of <= 512 products drained
                                   to float-float accumulators: error ~2^-28
                                   of (row max x column max) */
 #define CVSADC_FP64_SLICE7 3   /* as SLICE4 with seven slices (28 products):
@@ -264,8 +264,10 @@ int cvsadc_device_bytes(cvsadc_ctx* ctx, int64_t* bytes);
  */
 
 /* MP2 amplitudes, MP2 energy and (if tau > 0) the FNS truncation with the
- * rotation of B^P, then the M11 block and the transition moments.  The
- * dipole pointer may be NULL.  Section "Implementation and Computational
+ * rotation of B^P, then the M11 block and the transition moments.  In the
+ * tensor-core precisions a large rotation keeps 57 bits below the largest
+ * component of each row it contracts (FP64 in CVSADC_FP64).  The dipole
+ * pointer may be NULL.  Section "Implementation and Computational
  * Details", Eqs. 15 and 17-20. */
 int cvsadc_prepare(cvsadc_ctx* ctx, const cvsadc_params* params,
                    const double* eps, const void* B, const void* dip,
@@ -314,11 +316,12 @@ int cvsadc_sigma(cvsadc_ctx* ctx, int32_t precision, int32_t flags,
 /* Plain complex GEMM with the library's engines: C = A B for row-major
  * complex matrices A [M][lda], B [K][ldb], C [M][ldc] (interleaved
  * complex128).  precision CVSADC_FP64 runs the FP64 FMA kernel;
- * the mixed modes the tcgen05 kernels (see the precision constants) when
+ * the other modes the tcgen05 kernels (see the precision constants) when
  * the product is large enough to pay for its operand packing, else the
- * FP64 kernel.  Memory space per `flags`.  Errors:
- * EINVAL (sizes, leading dimensions), ETIMEOUT (a bounded device wait of
- * the tensor-core kernel expired), ENOMEM, ECUDA. */
+ * FP64 kernel (always for M N <= 4096, M + N <= 384 and K >= 4096).
+ * Memory space per `flags`.  Errors: EINVAL (sizes, leading dimensions),
+ * ETIMEOUT (a bounded device wait of the tensor-core kernel expired),
+ * ENOMEM, ECUDA. */
 int cvsadc_zgemm(cvsadc_ctx* ctx, int32_t precision, int32_t flags,
                  int32_t M, int32_t N, int32_t K, const void* A, int64_t lda,
                  const void* B, int64_t ldb, void* C, int64_t ldc);

@@ -558,13 +558,19 @@ void zgemm_tc(cudaStream_t s, int nprod, int M, int N, int K, double alpha,
 // scale 2^e with max |entry| < 2^e.  A scaled value a in (-1, 1) is cut into
 // integer slices q_i in [-128, 128] with a = sum_i q_i 2^{-7(i+1)} + r,
 // |r| <= 2^{-7 s - 1}; each slice is exactly a bf16.  A product of slices is
-// an integer with |q q'| <= 2^14, so a run of up to 1024 products sums
-// exactly in the FP32 tensor-memory accumulator (< 2^24).  Slice products
-// (i, j) with i + j <= s - 1 are kept and grouped so that a run never mixes
-// two (i, j) pairs; each finished run is drained from tensor memory (two
-// accumulator buffers, so draining overlaps the next run) and added, times
-// 2^{-7(i+j+2)}, to float-float accumulators (about 48 bits) in registers.
-// The epilogue applies 2^{e_m + f_n}, alpha and beta in FP64.
+// an integer with |q q'| <= 2^14, and short runs of them sum exactly in the
+// FP32 tensor-memory accumulator (up to 2^24; each kernel below counts its
+// own: 512 products on pairs of CTAs, 256 in the tile kernel).  Slice
+// products (i, j) with i + j <= s - 1 are kept; those of one order i + j
+// share an accumulator.  Each finished run is drained from tensor memory
+// while the next one is computed and added, times 2^{-7(i+j+2)}, to
+// accumulators in registers (float-float, about 48 bits; 8 slices: 64-bit
+// integers).  The epilogue applies 2^{e_m + f_n}, alpha and beta in FP64.
+//
+// The digits lie below a line's largest component, so a product is off by
+// about 2^(1 - 7 s) of row max x column max per term, whatever the size of
+// the term: small entries beside a large one are cut, and a line that holds
+// an infinity or a not-a-number gives infinities or not-a-numbers.
 //
 // ===========================================================================
 namespace {

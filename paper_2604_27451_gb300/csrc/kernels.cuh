@@ -35,8 +35,10 @@ void zgemm_tc(cudaStream_t s, int nprod, int M, int N, int K, double alpha,
 bool tc_available();
 // Exact-accumulation slice GEMM on the tensor cores (see gemm_tc.cu):
 // nslices = 4 (10 slice products, ~2^-28 of row max x column max), 7 (28
-// products, FP64 class) or 8 (36 products, no further from the exact sums
-// than FP64 arithmetic; no caches).
+// products, FP64 class) or 8 (36 products, ~2^-55 of row max x column max per
+// term: by norm no further from the exact sums than FP64 arithmetic where a
+// line's entries are of similar size, but small entries beside a large one
+// are cut, which FP64 keeps; no caches).
 // one bounded wait that expires after limit_ns (clamped to [1 ms, 4 s]) and
 // records its code in *err
 void wait_probe(cudaStream_t s, int64_t limit_ns, int* err);

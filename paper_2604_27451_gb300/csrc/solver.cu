@@ -380,7 +380,8 @@ void gemm64(cvsadc_ctx* c, int M, int N, int K, double alpha, View A,
             c->s_kpart.bytes / sizeof(cplx));
 }
 
-// C = A B with 8 slices: FP64 accuracy on the tensor cores
+// C = A B with 8 slices: 57 bits below the largest component of each row of A
+// and column of B, on the tensor cores
 void gemm_slice8(cvsadc_ctx* c, int M, int N, int K, View A, View B, View C) {
   A = checked(A);
   B = checked(B);
@@ -833,13 +834,15 @@ void build_fns(cvsadc_ctx* c, int prec, double tau) {
   // rotate B^P (and dipoles): occupied rows/cols unchanged, virtual with U
   const int n2 = o + vk;
   const int64_t nn = (int64_t)n * n, nn2 = (int64_t)n2 * n2;
-  // Slice precisions rotate with 8 slices (57 bits below a line's largest
-  // component, exact sums).  Against extended precision their error is 0.8e-16
-  // of the result's norm on 300 x 200 by 200 x 150 with Gaussian entries or a
-  // unitary factor, the FP64 kernels' 4.7e-16; and the FP64 pipes were the
-  // bound of this step: 1000 matrices of 246 x 246, 200 virtuals into 150:
-  // 99 -> 5.6 ms.  Small rotations stay on the FP64 kernels, by the rule of
-  // gemm().
+  // The tensor-core precisions rotate with 8 slices (57 bits below a line's
+  // largest component, exact sums); what they feed, the products of 4 or 7
+  // slices, keeps 2^-28 or 2^-49 of the same kind.  Against extended precision
+  // their error is 0.8e-16 of the result's norm on 300 x 200 by 200 x 150 with
+  // Gaussian entries or a unitary factor, the FP64 kernels' 4.7e-16 (by
+  // component FP64 keeps what is small beside the rest of its line, and these
+  // do not); and the FP64 pipes were the bound of this step: 1000 matrices of
+  // 246 x 246, 200 virtuals into 150: 99 -> 5.6 ms.  Small rotations stay on
+  // the FP64 kernels, by the rule of gemm().
   const bool slices = prec != CVSADC_FP64 && tc_available() && vk >= 32 && v >= 64;
   auto rotate = [&](const cplx* src, int64_t nmat, DBuf& dst) {
     dst.ensure((size_t)nmat * nn2 * sizeof(cplx));

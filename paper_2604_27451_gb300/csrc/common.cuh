@@ -214,6 +214,13 @@ void kstats_end(cudaStream_t s, int token);
 void kstats_collect(int kernel, int64_t* count, double* ms, double* flops);
 void kstats_reset();
 
+// How many of n items of `per` bytes fit in `have` bytes beside `fixed`: at
+// least one, also where `fixed` alone does not fit.
+static inline int64_t block_within(int64_t n, size_t fixed, size_t per, size_t have) {
+  const int64_t fit = have > fixed ? (int64_t)((have - fixed) / per) : 0;
+  return fit < 1 ? 1 : fit < n ? fit : n;
+}
+
 // ------------------------------------------------------------- launching
 static inline unsigned grid1d(int64_t n, int block, int64_t cap = 152 * 32) {
   int64_t g = (n + block - 1) / block;

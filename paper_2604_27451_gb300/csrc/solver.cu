@@ -858,8 +858,7 @@ void build_fns(cvsadc_ctx* c, int prec, double tau) {
       const size_t fixed = slice_workspace_bytes(0, vk, v, 8);
       const size_t per = slice_workspace_bytes(n, vk, v, 8) - fixed;
       const size_t have = std::min(ROT_PACK, std::max(c->s_tc.bytes, ROT_PACK / 16));
-      nb = have > fixed ? std::min<int64_t>(nmat, (int64_t)((have - fixed) / per)) : 1;
-      nb = std::max<int64_t>(1, nb);
+      nb = block_within(nmat, fixed, per, have);
     }
     DBuf tmp;
     tmp.ensure((size_t)nb * n * vk * sizeof(cplx));
